@@ -110,6 +110,12 @@ struct Hist {
         if (c)
             atomicAdd(hi + j, c);
     }
+    __device__ __forceinline__ void add32(int j, unsigned v) const
+    {
+        const unsigned old = atomicAdd(lo + j, v);
+        if (old + v < old)
+            atomicAdd(hi + j, 1u);
+    }
     __device__ __forceinline__ unsigned long long get(int j) const
     {
         return ((unsigned long long)hi[j] << 32) | lo[j];
@@ -148,6 +154,33 @@ struct RunAcc {
     }
 };
 
+// A 64-bit integer rounded to nearest in FP32 (as __ll2float_rn and
+// __float2ll_rn round, which run on the FP64 pipe, 64 cycles a warp
+// instruction): the top 32 bits with the bits below them as a sticky bit
+// round as the whole does.
+__device__ __forceinline__ float u64_to_float(unsigned long long v)
+{
+    const unsigned hi = (unsigned)(v >> 32);
+    if (hi == 0)
+        return __uint2float_rn((unsigned)v);
+    const int s = 32 - __clz((int)hi);  // 1..32
+    const unsigned w = (unsigned)(v >> s) | ((v << (64 - s)) ? 1u : 0u);
+    return __fmul_rn(__uint2float_rn(w), __uint_as_float((unsigned)(127 + s) << 23));
+}
+
+__device__ __forceinline__ float i64_to_float(long long v)
+{
+    const float f = u64_to_float((unsigned long long)(v < 0 ? -v : v));
+    return v < 0 ? -f : f;
+}
+
+__device__ __forceinline__ long long float_to_i64(float x)
+{
+    if (fabsf(x) < 2147483648.0f)
+        return __float2int_rn(x);
+    return __float2ll_rn(x);
+}
+
 __device__ __forceinline__ float span_to_float(long long span)
 {
     if ((unsigned long long)span < (1ull << 32))
@@ -155,32 +188,21 @@ __device__ __forceinline__ float span_to_float(long long span)
     return __fmaf_rn(__int2float_rn((int)(span >> 32)), 4294967296.0f, __uint2float_rn(frac_of(span)));
 }
 
-// floor(q 2^32 / span) for 0 <= q <= 2^28 and 2^32 < span < 2^46 (a particle
-// that crosses two or more cell edges): the whole-cell charge of a box
-// particle.  The float estimate (relative error below 2^-20, so within 256
-// of the quotient) is corrected once with the exact remainder and then by
-// at most two steps each way; the result is the exact integer floor, with
-// no 64-bit integer division.
-__device__ __forceinline__ long long div_q32(int q, long long span)
+// floor(q 2^32 / span) for 0 <= q <= 2^28 and 2^32 <= span < 2^46 (a particle
+// that covers whole cells): the whole-cell charge of a box particle, at most
+// q.  qf and inv are q and an approximate 1 / span in FP32.  The estimate's
+// relative error is below 2^-21, so it is within 130 of the quotient; the
+// exact remainder then gives the rest of it to the nearest integer (error
+// below 0.5 + 2^-14), and its sign the floor.  Only 32-bit conversions: the
+// 64-bit ones run on the FP64 pipe, 64 cycles a warp instruction.
+__device__ __forceinline__ unsigned whole_cell_charge(unsigned q, float qf, unsigned long long span, float inv)
 {
-    const long long num = (long long)q << 32;
-    float inv;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(span_to_float(span)));
-    long long P = __float2ll_rz(__fmul_rn(__fmul_rn(__int2float_rn(q), 4294967296.0f), inv));
-    long long r = num - P * span;
-    P += __float2ll_rn(__fmul_rn(__ll2float_rn(r), inv));
-    r = num - P * span;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (r < 0) {
-            P -= 1;
-            r += span;
-        } else if (r >= span) {
-            P += 1;
-            r -= span;
-        }
-    }
-    return P;
+    const unsigned P0 = __float2uint_rz(__fmul_rn(__fmul_rn(qf, 4294967296.0f), inv));
+    long long r = (long long)(((unsigned long long)q << 32) - (unsigned long long)P0 * span);
+    const float rf = __fmaf_rn(__int2float_rn((int)(r >> 32)), 4294967296.0f, __uint2float_rn((unsigned)r));
+    const int k = __float2int_rn(__fmul_rn(rf, inv));
+    r -= (long long)k * (long long)span;
+    return P0 + (unsigned)k - (r < 0 ? 1u : 0u);
 }
 
 // n whole cells starting at cell js (mod nx) each receive p units: +p at js
@@ -249,7 +271,7 @@ __device__ __forceinline__ void emit_cross(long long ua, int ja, long long ub, i
         return;
     }
     const long long nint = ncut - 1;
-    const long long P = div_q32(q, span);  // span > 2^32: two or more edges
+    const long long P = whole_cell_charge((unsigned)q, __int2float_rn(q), (unsigned long long)span, inv);
     const long long inner = nint * P;
     if ((long long)F > (long long)q - inner)
         F = (int)((long long)q - inner);
@@ -312,7 +334,7 @@ __device__ __forceinline__ void emit_first(long long ua, long long ub, int q, in
     long long F = __float2int_rn(__fmul_rn(__fmul_rn(df, inv), __int2float_rn(q)));
     F = min(max(F, 0ll), (long long)q);
     const long long nint = ncut - 1;
-    const long long P = nint > 0 ? div_q32(q, span) : 0;
+    const long long P = nint > 0 ? whole_cell_charge((unsigned)q, __int2float_rn(q), (unsigned long long)span, inv) : 0;
     const long long inner = nint * P;
     if (F > (long long)q - inner)
         F = (long long)q - inner;
@@ -364,88 +386,76 @@ __device__ __forceinline__ float pl_kappa(long long up, long long ua, long long 
     const long long ln = un > ub ? un - ub : ub - un;
     if (!(inc || dec) || lp == 0 || ls == 0 || ln == 0 || qs == 0)
         return 0.f;
-    const float fp = __ll2float_rn(lp), fs = __ll2float_rn(ls), fn = __ll2float_rn(ln);
+    const float fp = i64_to_float(lp), fs = i64_to_float(ls), fn = i64_to_float(ln);
     const float rp = __fdiv_rn(__int2float_rn(qp), fp);
     const float rs = __fdiv_rn(__int2float_rn(qs), fs);
     const float rn = __fdiv_rn(__int2float_rn(qn), fn);
     // twice the centroid distance c_{s+1} - c_{s-1}, signed
-    const float dc2 = __ll2float_rn((ub - up) + (un - ua));
+    const float dc2 = i64_to_float((ub - up) + (un - ua));
     const float k = __fdiv_rn(__fmul_rn(__fsub_rn(rn, rp), fs), __fmul_rn(rs, dc2));
     return fabsf(k) < 1e30f ? k : 0.f;
 }
 
-// Deposit one piecewise-linear particle shorter than the box (at most nx
-// cells, so the loop is bounded) that crosses at least one cell edge:
-// the cell between the cuts k and k+1 gets round(q phi(t_{k+1})) -
+// Piecewise-linear particles of a warp, one per lane (n cells of it, 0: none),
+// shorter than the box each.  From the lower end's cell jl, at the fraction la
+// of it, the cell between the cuts k and k+1 gets round(q phi(t_{k+1})) -
 // round(q phi(t_k)), phi(t) = t + kappa t (t - 1), t_k the fraction of the
 // length at the k-th edge (phi(0) = 0, phi(1) = 1), so the pieces sum to q
 // exactly.  A piece may be negative when |kappa| > 1 (the linear density
 // changes sign inside the particle).
-template <class ACC>
-__device__ __forceinline__ void emit_cross_linear(long long ua, int ja, long long ub, int jb, int q, float kappa,
-                                                  int nx, ACC &acc, unsigned &maxseg)
+//
+// The cells of all 32 particles are laid out one after another and dealt to
+// the lanes 32 at a time, each lane finding its particle in the running count
+// and taking its parameters from the owner: on folded sheets particles range
+// from two cells to half the box, and a loop per lane (or a warp per long
+// particle) left most lanes idle for a chain of divisions and conversions.
+// A step of 256 x 2048 folded tracers
+// on 256 cells takes 72 us, 120 us with those loops.
+__device__ __forceinline__ void emit_linear(int jl, unsigned la, float inv, int q, float kappa, int n, int nx,
+                                            const Hist &hist)
 {
-    if (ub < ua) {
-        const long long t = ua;
-        ua = ub;
-        ub = t;
-        const int tj = ja;
-        ja = jb;
-        jb = tj;
+    const int lane = threadIdx.x & 31;
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o)
+            incl += t;
     }
-    const long long span = ub - ua;
-    maxseg = max(maxseg, (unsigned)min((unsigned long long)span >> 16, 0xffffffffull));
-    const float inv = __frcp_rn(__ll2float_rn(span));
-    const float fq = __int2float_rn(q);
-    const long long ncut = (long long)cell_of(ub) - (long long)cell_of(ua);
-    const long long lo = (long long)frac_of(ua);
-    long long prev = 0;
-    int j = ja;
-    for (long long k = 1; k <= ncut; ++k) {
-        const float t = __fmul_rn(__ll2float_rn((k << 32) - lo), inv);
-        const float phi = __fmaf_rn(__fmul_rn(kappa, t), __fsub_rn(t, 1.0f), t);
-        const long long c = __float2ll_rn(__fmul_rn(fq, phi));
-        acc.add(j, c - prev);
-        prev = c;
-        j = (j + 1 == nx) ? 0 : j + 1;
-    }
-    acc.add(jb, (long long)q - prev);
-}
-
-// The same pieces as emit_cross_linear, with the particle's cells shared out
-// over the 32 lanes of the warp (all lanes call it with the same particle).
-template <class ACC>
-__device__ __forceinline__ void emit_linear_warp(long long ua, int ja, long long ub, int jb, int q, float kappa,
-                                                 int nx, ACC &acc, unsigned &maxseg, int lane)
-{
-    if (ub < ua) {
-        const long long t = ua;
-        ua = ub;
-        ub = t;
-        const int tj = ja;
-        ja = jb;
-        jb = tj;
-    }
-    const long long span = ub - ua;
-    maxseg = max(maxseg, (unsigned)min((unsigned long long)span >> 16, 0xffffffffull));
-    const float inv = __frcp_rn(__ll2float_rn(span));
-    const float fq = __int2float_rn(q);
-    const long long ncut = (long long)cell_of(ub) - (long long)cell_of(ua);
-    const long long lo = (long long)frac_of(ua);
-    auto cum = [&](long long k) -> long long {  // round(q phi(t_k)) at the k-th edge
-        const float t = __fmul_rn(__ll2float_rn((k << 32) - lo), inv);
-        const float phi = __fmaf_rn(__fmul_rn(kappa, t), __fsub_rn(t, 1.0f), t);
-        return __float2ll_rn(__fmul_rn(fq, phi));
-    };
-    for (long long k0 = 0; k0 <= ncut; k0 += 32) {
-        const long long k = k0 + lane;  // cell ja + k, between the edges k and k + 1
-        if (k <= ncut) {
-            const long long c_lo = k == 0 ? 0 : cum(k);
-            const long long c_hi = k == ncut ? (long long)q : cum(k + 1);
-            int j = ja + (int)k;  // k <= ncut <= nx
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    long long last = 0;  // round(q phi) at the upper cut of the cell before this pass's first
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        const int p = p0 + lane;
+        int own = 0;  // particles that end at or before p
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, own + o - 1) <= p)
+                own += o;
+        own = min(own, 31);  // past the end: any
+        const int n_o = __shfl_sync(0xffffffffu, n, own);
+        const int k = p - (__shfl_sync(0xffffffffu, incl, own) - n_o);  // cell jl + k
+        const int jl_o = __shfl_sync(0xffffffffu, jl, own);
+        const unsigned la_o = __shfl_sync(0xffffffffu, la, own);
+        const float inv_o = __shfl_sync(0xffffffffu, inv, own);
+        const float kap_o = __shfl_sync(0xffffffffu, kappa, own);
+        const int q_o = __shfl_sync(0xffffffffu, q, own);
+        long long up = q_o;  // round(q phi) at the cell's upper cut
+        if (k + 1 < n_o) {
+            const float t = __fmul_rn(u64_to_float(((unsigned long long)(unsigned)(k + 1) << 32) - la_o), inv_o);
+            const float phi = __fmaf_rn(__fmul_rn(kap_o, t), __fsub_rn(t, 1.0f), t);
+            up = float_to_i64(__fmul_rn(__int2float_rn(q_o), phi));
+        }
+        long long lo = __shfl_up_sync(0xffffffffu, up, 1);
+        if (lane == 0)
+            lo = last;
+        last = __shfl_sync(0xffffffffu, up, 31);
+        if (p < total) {
+            const long long piece = up - (k == 0 ? 0 : lo);
+            int j = jl_o + k;  // k <= nx
             if (j >= nx)
                 j -= nx;
-            acc.add(j, c_hi - c_lo);
+            if (piece)
+                hist.add(j, piece);
         }
     }
 }
@@ -512,15 +522,20 @@ __device__ __noinline__ Spill acc_spill(long long a, float y, unsigned long long
 }
 
 // Add y (a term already in the sum's fixed-point unit), truncated to an
-// integer, to a lane's 64-bit sum.  A term of 2^62 or more, or one that
-// would overflow the sum, takes the rare path, which moves the lane's sum
-// into the block's 128-bit sum: the total stays exact, so it does not
-// depend on the order of the additions.
+// integer, to a lane's 64-bit sum.  Below 2^53 the integer is the exact sum
+// of two 32-bit conversions, y's multiple of 2^22 and the rest (both exact in
+// FP32: y has 24 bits); one 64-bit conversion would take the FP64 pipe 64
+// cycles a warp.  A term of 2^53 or more, or one that would overflow the sum,
+// takes the rare path, which moves the lane's sum into the block's 128-bit
+// sum: the total stays exact, so it does not depend on the order of the
+// additions.
 __device__ __forceinline__ void sum_add(long long &a, float y, unsigned long long *blk, unsigned &err)
 {
-    const long long v = __float2ll_rz(y);
+    const int h = __float2int_rz(__fmul_rn(y, 0x1p-22f));
+    const int l = __float2int_rz(__fmaf_rn(__int2float_rn(h), -0x1p22f, y));
+    const long long v = (long long)h * (1ll << 22) + l;
     const long long s = (long long)((unsigned long long)a + (unsigned long long)v);
-    if (__builtin_expect(!(fabsf(y) < 4611686018427387904.0f) || ((a ^ s) & (v ^ s)) < 0, 0)) {
+    if (__builtin_expect(!(fabsf(y) < 9007199254740992.0f) || ((a ^ s) & (v ^ s)) < 0, 0)) {
         const Spill r = acc_spill(a, y, blk);
         a = r.a;
         err |= r.err;
@@ -606,13 +621,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsig
 constexpr int kStageBytesU = SIC_STAGE_U_BYTES;
 constexpr int kStageBytesV = SIC_STAGE_V_BYTES;
 constexpr int kStageBytesQ = SIC_STAGE_Q_BYTES;
+// the box deposit's table of a warp's positions (and as much again of running
+// charges), entry r of lane l at 32 r + l, r = 0..R
+constexpr int kTabWords = 32 * (SIC_K1_R + 1);
+constexpr int kTabBytes = 4 * kTabWords;
 
 // Per-warp buffer: two stages when staging (U | V | Q each), otherwise one
 // scratch of new positions (U | Q) for the cross-cell pass.
 template <bool PER_Q, bool STAGED>
 struct WarpBuf {
     static constexpr int q_offset = STAGED ? kStageBytesU + kStageBytesV : kStageBytesU;
-    static constexpr int stage = q_offset + (PER_Q ? kStageBytesQ : 0);
+    // (without staging the box deposit's table is the larger use)
+    static constexpr int stage = STAGED ? q_offset + (PER_Q ? kStageBytesQ : 0) : (PER_Q ? 2 : 1) * kTabBytes;
+    static_assert(stage >= (PER_Q ? 2 : 1) * kTabBytes && stage >= q_offset + (PER_Q ? kStageBytesQ : 0),
+                  "a stage holds the item and the table");
     static constexpr int bytes = (STAGED ? 2 : 1) * stage;
 };
 
@@ -681,7 +703,6 @@ struct Shared {
 };
 
 constexpr size_t kSharedHead = (sizeof(Shared) + 15) / 16 * 16;
-constexpr int kWarpCuts = 8;  // piecewise-linear particles this many cells long use the whole warp
 
 // shared head, mesh lo/hi [nx], diff [nx + 2], kick pairs [nx] (float2);
 // staging starts on a 128-byte boundary (bulk copies need 16)
@@ -1017,6 +1038,146 @@ __device__ void add_diff_prefix(const Hist &hist, const Hist &diff, int nx, Shar
 
 // ---------------------------------------------------------------- kernel ----
 
+// The box deposit of one warp's tracers, R consecutive ones per lane at u with
+// cells jn (nu, nj, nq: the tracer after the lane's last one; nseg: segments
+// starting at the lane's tracers, nseg_item: at the item's).
+//
+// Along a lane, charge is carried in `pend` until the sheet leaves the cell it
+// is in: a segment inside a cell adds its charge to it, one that crosses edges
+// commits it together with its share of the cell it leaves and carries on with
+// its share of the cell it arrives in.  So a lane makes one commit per crossing
+// segment and one at its end, and the crossing segments of the lanes are dealt
+// with side by side: the loop runs as often as the lane with the most of them
+// asks (once on quiet sheets).  With one charge per sheet, lanes without a
+// crossing make no commit: the lane with a crossing before them takes their
+// segments into its last one (they lie in one cell), which also spares
+// the adds of many lanes into one word.  No list of the crossing ones is made
+// and no lane works for another.  Against per-cell counts and a warp-wide task
+// list for the crossing ones (us per step, before and after): 4.2 M folded
+// tracers 72 and 60, 2.3 M folded 50 and 43, 8.4 M quiet 43 and 41; a batch of
+// 66 M quiet 278 and 254.
+//
+// A crossing segment of q units in 32.32 cell coordinates: its lower end's
+// cell gets F = round(q (e_1 - a) / (b - a)) (FP32, approximate reciprocal,
+// clamped), every whole cell inside P = floor(q 2^32 / (b - a)), the upper
+// end's the rest: all below 2^28, so the arithmetic is 32 bits wide.
+// tab: the lane's positions (and running charges) by index, entry r of lane l
+// at 32 r + l, so that a lane's own choice of r never conflicts.
+template <bool PER_Q, bool FULL>
+__device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int (&jn)[R], const int (&q)[R], unsigned nu,
+                                              int nj, int nq, int nseg, int rn, int nseg_item, int qs_sheet, int segq,
+                                              int nx, const Hist &hist, const Hist &diff, int *diff_used, unsigned *tab,
+                                              unsigned &mlen)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned nx4 = (unsigned)nx << SIC_POS_WIND_BITS;
+    unsigned cross = 0;
+    unsigned qsum = 0;  // per-tracer charges: of the segments before r
+    __syncwarp();       // every lane has read its tracers: the table takes their place
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const bool end = FULL ? r + 1 == R : r + 1 >= rn;  // the next tracer is the one after the lane's
+        const unsigned ub = end ? nu : u[r + 1 < R ? r + 1 : r];
+        const int jb = end ? nj : jn[r + 1 < R ? r + 1 : r];
+        // inside one cell: both ends in it and shorter than half a box (a
+        // longer one could end in the same cell one box on)
+        const bool in = jb == jn[r] && (ub - u[r] + (1u << 29)) < (1u << 30);
+        const bool seg = (FULL && r + 1 < R) || r < nseg;
+        if (seg && !in)
+            cross |= 1u << r;
+        if (PER_Q) {
+            const int qb = end ? nq : q[r + 1 < R ? r + 1 : r];
+            tab[kTabWords + 32 * r + lane] = qsum;
+            qsum += seg ? (unsigned)(segq ? q[r] : q[r] + qb) : 0u;
+        }
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, cross != 0);
+    unsigned pend = 0;  // charge waiting for cell c (below 2^32: at most 9 shares of 2^28)
+    int c = jn[0];
+    int done = 0;       // segments of the lane dealt with
+    if (who) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            tab[32 * r + lane] = u[r];
+        if (FULL || rn == R) {
+            tab[32 * R + lane] = nu;
+        } else if (rn > 0) {
+#pragma unroll
+            for (int r = 1; r < R; ++r)
+                if (r == rn)
+                    tab[32 * r + lane] = nu;
+        }
+        if (PER_Q)
+            tab[kTabWords + 32 * R + lane] = qsum;
+        while (cross) {
+            const int k = __ffs(cross) - 1;
+            cross &= cross - 1u;
+            const unsigned pa = tab[32 * k + lane], pb = tab[32 * k + 32 + lane];
+            unsigned qs, before;
+            if (PER_Q) {
+                const unsigned q0 = tab[kTabWords + 32 * k + lane], q1 = tab[kTabWords + 32 * k + 32 + lane];
+                qs = q1 - q0;
+                before = q0 - tab[kTabWords + 32 * done + lane];
+            } else {
+                qs = (unsigned)qs_sheet;
+                before = (unsigned)(k - done) * qs;
+            }
+            done = k + 1;
+            const int cb = cell_of(cell_coord(pb, nx));
+            const int d = (int)(pb - pa);
+            const bool back = d < 0;
+            const unsigned len = (unsigned)abs(d);
+            mlen = max(mlen, len);
+            const unsigned la = (back ? pb : pa) * nx4;  // the lower end's fraction of its cell
+            const unsigned long long span = (unsigned long long)len * nx4;
+            const float df = la ? __uint2float_rn(0u - la) : 4294967296.0f;  // to the first edge
+            const float sf = __fmaf_rn(__int2float_rn((int)(span >> 32)), 4294967296.0f, __uint2float_rn((unsigned)span));
+            // an approximate reciprocal is enough: F is clamped to [0, q] and
+            // the other end takes the rest, so the charge stays exact
+            float inv;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(sf));
+            const float qf = __int2float_rn((int)qs);
+            unsigned F = (unsigned)min(max(__float2int_rn(__fmul_rn(__fmul_rn(df, inv), qf)), 0), (int)qs);
+            const int nint = (int)((span + la) >> 32) - 1;  // whole cells inside
+            unsigned inner = 0;
+            if (nint > 0) {
+                const unsigned P = whole_cell_charge(qs, qf, span, inv);
+                inner = (unsigned)nint * P;  // at most qs
+                F = min(F, qs - inner);
+                int js = (back ? cb : c) + 1;
+                js = js == nx ? 0 : js;
+                if (nint <= 2) {
+                    hist.add32(js, P);
+                    if (nint == 2)
+                        hist.add32(js + 1 == nx ? 0 : js + 1, P);
+                } else {
+                    range_add(js, nint, (long long)P, nx, diff, diff_used);
+                }
+            }
+            const unsigned rest = qs - F - inner;
+            hist.add32(c, pend + before + (back ? rest : F));
+            pend = back ? F : rest;
+            c = cb;
+        }
+    }
+    // what is left of the lane, in the cell its sheet is in now
+    if (PER_Q) {
+        const unsigned left = pend + (qsum - (done ? tab[kTabWords + 32 * done + lane] : 0u));
+        if (left)
+            hist.add32(c, left);
+    } else {
+        const unsigned owners = who | 1u;
+        if ((owners >> lane) & 1u) {
+            const unsigned above = owners & (0xfffffffeu << lane);           // the lanes with a crossing after this one
+            const int upto = above ? R * (__ffs(above) - 1) : nseg_item;     // (the first of them; the item's end)
+            const int mine = min(upto, nseg_item) - (lane * R + done);
+            const unsigned long long left = pend + (unsigned long long)(unsigned)max(mine, 0) * (unsigned)qs_sheet;
+            if (left)
+                hist.add(c, (long long)left);
+        }
+    }
+}
+
 // One work item (up to 32 R tracers, R per lane) of the current simulation.
 // FULL: the item has all 32 R tracers, so no lane needs a bounds test.
 template <bool PUSH, bool DEPOSIT, bool PER_Q, bool FULL, bool STAGED, bool GEN, class MID>
@@ -1025,7 +1186,7 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
                                         float *__restrict__ Vout, const int32_t *__restrict__ Qh,
                                         const float2 *ek, const Hist &hist, const Hist &diff,
                                         Shared &sh, int nx, float ks, int drift, unsigned &rerr,
-                                        char *st, unsigned short *tasks, long long &ake, long long &ap, unsigned &mseg,
+                                        char *st, unsigned short *tasks, long long &ake, long long &ap, unsigned &mseg, unsigned &mlen,
                                         const WorkItemPL *pw, int dep, int segq, bool track_all, const MID &mid)
 {
     const unsigned *stU = reinterpret_cast<const unsigned *>(st);
@@ -1228,6 +1389,32 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
             }
         }
         run.flush();
+    } else if (DEPOSIT && !(GEN && (pw != nullptr || dep == SIC_DEPOSIT_FIRST))) {
+        hu += W.halo_shift;  // closing segment: the sheet's first tracer one winding on
+        // the tracer after each lane's last one: the next lane's first, or the halo
+        unsigned nu = __shfl_down_sync(0xffffffffu, u[0], 1);
+        int nj = __shfl_down_sync(0xffffffffu, jn[0], 1);
+        int nq = __shfl_down_sync(0xffffffffu, q[0], 1);
+        int nseg = rn;  // segments that start at this lane's tracers
+        if (lane >= lane_last) {
+            nu = hu;
+            nj = hj;
+            nq = hq;
+            if (lane == lane_last && !has_halo)
+                --nseg;
+        }
+        deposit_boxes<PER_Q, FULL>(u, jn, q, nu, nj, nq, nseg, rn, m - (W.halo >= 0 ? 0 : 1), 2 * W.qh, segq, nx,
+                                   hist, diff, &sh.diff_used, reinterpret_cast<unsigned *>(st), mlen);
+        if (track_all) {
+            // a refinement length shorter than a cell: particles inside one
+            // cell count towards the longest one too
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (r < nseg) {
+                    const unsigned ub = (r + 1 < R && r + 1 < rn) ? u[r + 1 < R ? r + 1 : r] : nu;
+                    mlen = max(mlen, (unsigned)abs((int)(ub - u[r])));
+                }
+        }
     } else if (DEPOSIT) {
         hu += W.halo_shift;  // closing segment: the sheet's first tracer one winding on
         // publish the new positions (and charges) of the item in shared
@@ -1423,23 +1610,7 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
             mseg = max(mseg, (unsigned)min(((unsigned long long)longest * (unsigned)nx4) >> 16, 0xffffffffull));
         }
 
-        // cross-cell segments of box particles, at most one per lane (the
-        // usual case): each lane deposits its own
-        const int cnt = __popc(cross);
-        const bool boxes = !(GEN && pw != nullptr);
-        if (boxes && !__any_sync(0xffffffffu, cnt > 1)) {
-            if (cross) {
-                const int idx = l0 + __ffs(cross) - 1;
-                const unsigned pa = pts[idx], pb = pts[idx + 1];
-                const long long ua = cell_coord(pa, nx);
-                const long long ub = ua + seg_span(pa, pb, nx4);
-                const int qs = PER_Q ? qpts[idx] + (segq ? 0 : qpts[idx + 1]) : qs_sheet;
-                DirectAdd acc{hist};
-                emit_cross(ua, cell_of(ua), ub, cell_of(cell_coord(pb, nx)), qs, nx, acc, diff, &sh.diff_used, mseg);
-            }
-            cross = 0;
-        }
-        // the others: compact them into a task list and let every lane take
+        // cross-cell segments: compact them into a task list and let every lane take
         // one in turn; a lane's slot is the count before it, summed from one
         // ballot per bit of the per-lane counts (0..R) when there are any
         unsigned lt;
@@ -1481,46 +1652,32 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
                 const int qn = PER_Q ? qpts[idx + 1] + (segq ? 0 : qpts[idx + 2]) : qs_sheet;
                 return pl_kappa(up, ua, ub, un, qp, qs, qn);
             };
-            bool any_long = false;
-            for (int k = lane; k < total; k += 32) {
-                const int idx = tasks[k];
-                const unsigned pa = pts[idx], pb = pts[idx + 1];
-                const long long ua = cell_coord(pa, nx);
-                const long long ub = ua + seg_span(pa, pb, nx4);
-                const int ja = cell_of(ua), jb = cell_of(cell_coord(pb, nx));
-                const int qs = PER_Q ? qpts[idx] + (segq ? 0 : qpts[idx + 1]) : qs_sheet;
-                const float kappa = (GEN && pw != nullptr) ? kappa_of(idx, ua, ub, qs) : 0.f;
-                if (kappa == 0.f) {
-                    emit_cross(ua, ja, ub, jb, qs, nx, acc, diff, &sh.diff_used, mseg);
-                } else {
-                    const int cuts = cell_of(ua) > cell_of(ub) ? cell_of(ua) - cell_of(ub) : cell_of(ub) - cell_of(ua);
-                    if (cuts >= kWarpCuts) {
-                        tasks[k] = (unsigned short)(idx | 0x8000);  // for the whole warp, below
-                        any_long = true;
+            for (int k0 = 0; k0 < total; k0 += 32) {
+                const int k = k0 + lane;
+                int jl = 0, qs = 0, n = 0;
+                unsigned la = 0u;
+                float inv = 0.f, kappa = 0.f;
+                if (k < total) {
+                    const int idx = tasks[k];
+                    const unsigned pa = pts[idx], pb = pts[idx + 1];
+                    const long long ua = cell_coord(pa, nx);
+                    const long long ub = ua + seg_span(pa, pb, nx4);
+                    qs = PER_Q ? qpts[idx] + (segq ? 0 : qpts[idx + 1]) : qs_sheet;
+                    kappa = kappa_of(idx, ua, ub, qs);
+                    const int ja = cell_of(ua), jb = cell_of(cell_coord(pb, nx));
+                    if (kappa == 0.f) {
+                        emit_cross(ua, ja, ub, jb, qs, nx, acc, diff, &sh.diff_used, mseg);
                     } else {
-                        emit_cross_linear(ua, ja, ub, jb, qs, kappa, nx, acc, mseg);
+                        const long long lo = min(ua, ub), span = max(ua, ub) - lo;
+                        mseg = max(mseg, (unsigned)min((unsigned long long)span >> 16, 0xffffffffull));
+                        jl = ub < ua ? jb : ja;
+                        la = frac_of(lo);
+                        inv = __frcp_rn(u64_to_float((unsigned long long)span));
+                        n = cell_of(max(ua, ub)) - cell_of(lo) + 1;
                     }
                 }
-            }
-            // long piecewise-linear particles: every lane takes some of the
-            // particle's cells (the pieces do not depend on who computes them)
-            if (GEN && pw != nullptr && __any_sync(0xffffffffu, any_long)) {
                 __syncwarp();
-                for (int base = 0; base < total; base += 32) {
-                    const int k = base + lane;
-                    unsigned bal = __ballot_sync(0xffffffffu, k < total && (tasks[k] & 0x8000));
-                    while (bal) {
-                        const int src = __ffs(bal) - 1;
-                        bal &= bal - 1u;
-                        const int idx = tasks[base + src] & 0x7fff;
-                        const unsigned pa = pts[idx], pb = pts[idx + 1];
-                        const long long ua = cell_coord(pa, nx);
-                        const long long ub = ua + seg_span(pa, pb, nx4);
-                        const int qs = PER_Q ? qpts[idx] + (segq ? 0 : qpts[idx + 1]) : qs_sheet;
-                        emit_linear_warp(ua, cell_of(ua), ub, cell_of(cell_coord(pb, nx)), qs,
-                                         kappa_of(idx, ua, ub, qs), nx, acc, mseg, lane);
-                    }
-                }
+                emit_linear(jl, la, inv, qs, kappa, n, nx, hist);
             }
         }
         }  // not first-order
@@ -1584,6 +1741,7 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
         cur = lo;
     }
     unsigned rerr = 0, mseg = 0;
+    unsigned mlen = 0;  // longest crossing box particle, position units
     long long ake = 0, ap = 0;  // this lane's KE and P sums (units 2^-ke_u, 2^-p_u)
     bool first = true;          // the block's first simulation of the launch
     bool triggered = false;     // the next launch in the stream may start
@@ -1737,11 +1895,11 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
                     char *st = my_stage + s * WarpBuf<PER_Q, true>::stage;
                     if (W.count == WT)
                         do_item<PUSH, DEPOSIT, PER_Q, true, true, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                  nx, ks, drift, rerr, st, tasks, ake, ap, mseg, plw,
+                                                                  nx, ks, drift, rerr, st, tasks, ake, ap, mseg, mlen, plw,
                                                                   S.deposit, S.seg_q, track_all, mid);
                     else
                         do_item<PUSH, DEPOSIT, PER_Q, false, true, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                   nx, ks, drift, rerr, st, tasks, ake, ap, mseg, plw,
+                                                                   nx, ks, drift, rerr, st, tasks, ake, ap, mseg, mlen, plw,
                                                                    S.deposit, S.seg_q, track_all, mid);
                     __syncwarp();
                     s ^= 1;
@@ -1749,11 +1907,11 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
                     auto mid = []() {};
                     if (W.count == WT)
                         do_item<PUSH, DEPOSIT, PER_Q, true, false, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                   nx, ks, drift, rerr, my_stage, tasks, ake, ap, mseg,
+                                                                   nx, ks, drift, rerr, my_stage, tasks, ake, ap, mseg, mlen,
                                                                    plw, S.deposit, S.seg_q, track_all, mid);
                     else
                         do_item<PUSH, DEPOSIT, PER_Q, false, false, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                    nx, ks, drift, rerr, my_stage, tasks, ake, ap, mseg,
+                                                                    nx, ks, drift, rerr, my_stage, tasks, ake, ap, mseg, mlen,
                                                                     plw, S.deposit, S.seg_q, track_all, mid);
                 }
             }
@@ -1788,6 +1946,8 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
             ap = 0;
         }
         if (DEPOSIT) {
+            mseg = max(mseg, (unsigned)(((unsigned long long)mlen * (unsigned)(nx << SIC_POS_WIND_BITS)) >> 16));
+            mlen = 0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
                 mseg = max(mseg, __shfl_down_sync(0xffffffffu, mseg, o));
