@@ -273,7 +273,8 @@ int sic_push(sic_sim *sim);
  * by the sheet deposit of Eq. overlap and Eq. rho_sum): gather and push with
  * the current field, deposit every particle of the new positions, solve the
  * field (Sec. 2.1).  Each step is one kernel launch, the field solved by the
- * block that finishes last; runs of 8 steps replay a captured CUDA graph.
+ * grid that stays resident); on a stream that is being captured, and for meshes
+ * too large for that, one launch a step (runs of 8 replay a captured graph).
  * n_steps >= 0.  Asynchronous on the simulation's stream: errors found on
  * the device are returned by the next synchronising call (sic_sync,
  * sic_diagnostics, ...).  A held simulation (an error, or a particle past

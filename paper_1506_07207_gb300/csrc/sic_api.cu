@@ -428,6 +428,32 @@ void free_plan(Plan &p, cudaStream_t s)
     p.mem = nullptr;
 }
 
+// A simulation of this many items or fewer runs on one block, its mesh in
+// shared memory: two items a warp cost less than adding two blocks' meshes
+// through L2 and waiting (16 items, 64 cells: 6.2 us a step on one block, 6.8
+// on two).
+constexpr int kOneBlockItems = 16;
+
+// The groups of blocks of a launch of many steps (k_run), one per simulation:
+// block_begin[slot], and the grid; 0 when the steps are better launched one
+// by one.
+static int split_blocks(sic_sim *const *sims, int n, int nx_max, bool per_q, bool gen, std::vector<int32_t> &block_begin)
+{
+    const int per_sm = run_blocks_per_sm(nx_max, per_q, gen);
+    const int most = env_int("SIC_GRID", num_sms() * per_sm);  // (the test knob of build_plan)
+    if (per_sm < 1 || n != 1)
+        return 0;
+    block_begin.assign(n + 1, 0);
+    for (int slot = 0; slot < n; ++slot) {
+        const int items = (int)sims[slot]->items.size();
+        int blocks = (items + SIC_K1_WARPS - 1) / SIC_K1_WARPS;
+        if (items <= kOneBlockItems)
+            blocks = 1;
+        block_begin[slot + 1] = block_begin[slot] + std::max(1, std::min({blocks, most, num_sms() * per_sm}));
+    }
+    return block_begin[n];
+}
+
 // Build the device plan of one launch over several simulations (slot order):
 // the table of their descriptors, where each one's items start in the
 // launch's list, and the zeroed claim cursors, item tickets and block count.
@@ -464,10 +490,18 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     // simulation that all of them share is 1/D of its fair share, and a small
     // simulation is spread over many warps (D = SIC_CLAIM_DIV, default 4)
     const float claim_q = (float)(1.0 / ((double)env_int("SIC_CLAIM_DIV", 4) * grid * SIC_K1_WARPS));
+    bool gen = false;
+    for (int slot = 0; slot < n; ++slot)
+        gen = gen || sims[slot]->deposit != SIC_DEPOSIT_BOX;
+    std::vector<int32_t> block_begin;
+    p.run_grid = split_blocks(sims, n, nx_max, per_q, gen, block_begin);
     Layout lay;
     const size_t oT = lay.take(sizeof(SimDev) * table.size());
     const size_t oS = lay.take(4 * slot_begin.size());
+    const size_t oB = p.run_grid ? lay.take(4 * block_begin.size()) : 0;
     const size_t oK = lay.take(4 * (size_t)(2 * n + 1));  // cursor[n], tickets[n], done
+    const size_t oC = p.run_grid ? lay.take(sizeof(RunCtl) * (size_t)n) : lay.off;
+    const size_t cleared = lay.off - oK;
     cudaError_t e = cudaMallocAsync(&p.mem, lay.off, s);
     if (e != cudaSuccess)
         return e;
@@ -475,8 +509,10 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     e = cudaMemcpyAsync(b + oT, table.data(), sizeof(SimDev) * table.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b + oS, slot_begin.data(), 4 * slot_begin.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && p.run_grid)
+        e = cudaMemcpyAsync(b + oB, block_begin.data(), 4 * block_begin.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(b + oK, 0, 4 * (size_t)(2 * n + 1), s);
+        e = cudaMemsetAsync(b + oK, 0, cleared, s);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(s);  // host staging vectors go out of scope
     if (e != cudaSuccess)
@@ -491,11 +527,10 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     p.args.claim_min = 1;
     p.args.n_slots = n;
     p.args.nx_max = nx_max;
-    p.args.gen = 0;
-    for (int slot = 0; slot < n; ++slot)
-        p.args.gen |= sims[slot]->deposit != SIC_DEPOSIT_BOX ? 1 : 0;
+    p.args.gen = gen ? 1 : 0;
     p.grid = grid;
     p.per_q = per_q;
+    p.run = RunArgs{p.args.sims, (const int32_t *)(b + oB), (RunCtl *)(b + oC), n, nx_max, 0};
     return cudaSuccess;
 }
 
@@ -504,6 +539,31 @@ void set_schedule(Plan &p, int claim_div, int staging, int claim_min)
     p.args.claim_q = (float)(1.0 / ((double)std::max(1, claim_div) * p.grid * SIC_K1_WARPS));
     p.args.staging = staging;
     p.args.claim_min = std::max(1, claim_min);
+}
+
+constexpr int kStepsALaunch = 256;
+
+bool launch_many(Plan &p, int n_steps, cudaStream_t s, cudaError_t &e)
+{
+    e = cudaSuccess;
+    if (!p.run_grid || n_steps < 2)
+        return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return false;
+    for (int left = n_steps; left > 0 && e == cudaSuccess;) {
+        RunArgs a = p.run;
+        a.n_steps = std::min(left, kStepsALaunch);
+        e = launch_run_kernel(a, p.run_grid, p.per_q, p.args.gen != 0, s);
+        if (left == n_steps && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
+            cudaGetLastError();  // not on this device: one launch a step from now on
+            e = cudaSuccess;
+            p.run_grid = 0;
+            return false;
+        }
+        left -= a.n_steps;
+    }
+    return true;
 }
 
 cudaError_t launch(const Plan &p, Mode mode, float kick_scale, int drift, int record, cudaStream_t s)
@@ -1001,6 +1061,11 @@ int sic_step(sic_sim *sim, int32_t n_steps)
 {
     if (!sim || n_steps < 0)
         return SIC_EINVAL;
+    {
+        cudaError_t e;
+        if (launch_many(sim->plan, n_steps, sim->stream, e))
+            return e == cudaSuccess ? SIC_OK : fail_cuda(sim, e);
+    }
     if (n_steps >= kGraphSteps && !sim->gexec) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(sim->stream, cudaStreamCaptureModeThreadLocal));

@@ -18,6 +18,8 @@ struct Plan {
     LaunchArgs args{};
     int grid = 0;
     bool per_q = false;
+    RunArgs run{};       // many steps in one launch (run_grid 0: not for this plan)
+    int run_grid = 0;
 };
 
 // Device bytes of one simulation's allocation (state, meshes, items, ...).
@@ -86,4 +88,8 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s);
 void set_schedule(Plan &p, int claim_div, int staging, int claim_min);
 void free_plan(Plan &p, cudaStream_t s);
 cudaError_t launch(const Plan &p, sic::Mode mode, float kick_scale, int drift, int record, cudaStream_t s);
+// n_steps steps of the plan in launches of many steps each; false (and nothing
+// launched) when they have to be launched one by one: the plan is not for it,
+// the stream is being captured, or the device will not hold the whole grid.
+bool launch_many(Plan &p, int n_steps, cudaStream_t s, cudaError_t &e);
 }  // namespace sic_host

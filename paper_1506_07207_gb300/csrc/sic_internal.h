@@ -179,10 +179,34 @@ struct LaunchArgs {
                                  // 1: never; 2: whenever it fits (autotuning)
 };
 
+// What the blocks of one simulation share in a launch of k_run (all zero
+// between launches): the sums of three steps (SimAccum::pad[0]: error bits)
+// and the counts of blocks that have finished a step and that have left.
+struct RunCtl {
+    SimAccum acc[3];
+    unsigned bar;
+    unsigned out;
+    unsigned pad[30];
+};
+
+// One launch of k_run: n_steps steps of every simulation.
+struct RunArgs {
+    const SimDev *sims;          // table, one entry per slot
+    const int32_t *block_begin;  // [slots + 1] first block of each slot's group
+    RunCtl *ctl;                 // [slots]
+    int32_t n_slots;
+    int32_t nx_max;
+    int32_t n_steps;
+};
+
 #include <cuda_runtime.h>
 namespace sic {
 enum Mode { MODE_STEP = 0, MODE_DEPOSIT = 1, MODE_PUSH = 2 };
 cudaError_t launch_step_kernel(const LaunchArgs &a, int grid, Mode mode, bool per_q, cudaStream_t s);
+// Many steps in one cooperative launch; the blocks of it an SM holds (0: the
+// meshes are too large for it)
+cudaError_t launch_run_kernel(const RunArgs &a, int grid, bool per_q, bool gen, cudaStream_t s);
+int run_blocks_per_sm(int nx_max, bool per_q, bool gen);
 cudaError_t launch_field_out(const SimDev &sim, cudaStream_t s);
 cudaError_t launch_spectrum(const SimDev &sim, int field, cudaStream_t s);
 cudaError_t launch_refine_count(const SimDev &sim, long long lfix, int32_t *splits, cudaStream_t s);
