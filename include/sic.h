@@ -272,9 +272,10 @@ int sic_push(sic_sim *sim);
  * n_steps full SIC steps (Sec. 2.3: the PIC cycle with the scatter replaced
  * by the sheet deposit of Eq. overlap and Eq. rho_sum): gather and push with
  * the current field, deposit every particle of the new positions, solve the
- * field (Sec. 2.1).  Each step is one kernel launch, the field solved by the
- * grid that stays resident); on a stream that is being captured, and for meshes
- * too large for that, one launch a step (runs of 8 replay a captured graph).
+ * field (Sec. 2.1).  Two steps or more are taken many to a kernel launch (a
+ * cooperative grid that stays resident); a single step, steps on a stream that
+ * is being captured and meshes too large for that take one launch a step, runs
+ * of 8 in a replayed graph.
  * n_steps >= 0.  Asynchronous on the simulation's stream: errors found on
  * the device are returned by the next synchronising call (sic_sync,
  * sic_diagnostics, ...).  A held simulation (an error, or a particle past

@@ -116,6 +116,11 @@ struct Hist {
         if (old + v < old)
             atomicAdd(hi + j, 1u);
     }
+    __device__ __forceinline__ void sub32(int j, unsigned v) const  // v > 0
+    {
+        if (atomicAdd(lo + j, 0u - v) < v)
+            atomicAdd(hi + j, 0xffffffffu);
+    }
     __device__ __forceinline__ unsigned long long get(int j) const
     {
         return ((unsigned long long)hi[j] << 32) | lo[j];
@@ -1059,8 +1064,9 @@ __device__ void add_diff_prefix(const Hist &hist, const Hist &diff, int nx, Shar
 // the adds of many lanes into one word.  No list of the crossing ones is made
 // and no lane works for another.  Against per-cell counts and a warp-wide task
 // list for the crossing ones (us per step, before and after): 4.2 M folded
-// tracers 72 and 60, 2.3 M folded 50 and 43, 8.4 M quiet 43 and 41; a batch of
-// 66 M quiet 278 and 254.
+// tracers 72 and 51, 2.3 M folded 50 and 34, 8.4 M quiet 43 and 41; a batch of
+// 66 M quiet 278 and 246.  (With the whole cells through the general
+// range_add, a call of 64-bit adds: 60, 42.)
 //
 // A crossing segment of q units in 32.32 cell coordinates: its lower end's
 // cell gets F = round(q (e_1 - a) / (b - a)) (FP32, approximate reciprocal,
@@ -1151,12 +1157,22 @@ __device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int 
                 F = min(F, qs - inner);
                 int js = (back ? cb : c) + 1;
                 js = js == nx ? 0 : js;
-                if (nint <= 2) {
-                    hist.add32(js, P);
-                    if (nint == 2)
-                        hist.add32(js + 1 == nx ? 0 : js + 1, P);
-                } else {
+                if (nint >= nx) {
                     range_add(js, nint, (long long)P, nx, diff, diff_used);
+                } else if (P) {
+                    // one cell: into the mesh; more: +P at the first and -P
+                    // after the last in the difference array
+                    const Hist to{nint > 1 ? diff.lo : hist.lo, nint > 1 ? diff.hi : hist.hi};
+                    to.add32(js, P);
+                    if (nint > 1) {
+                        int je = js + nint;
+                        if (je > nx) {
+                            diff.add32(0, P);
+                            je -= nx;
+                        }
+                        diff.sub32(je, P);
+                        *diff_used = 1;
+                    }
                 }
             }
             const unsigned rest = qs - F - inner;
@@ -2134,8 +2150,8 @@ __device__ __forceinline__ bool group_wait(const unsigned *bar, unsigned target)
 // k_field_out writes on request, serve as the second and third mesh.
 //
 // us per step in runs of 160 steps, graphs of single steps and this: 4 K
-// tracers 9.8 and 6.2, 262 K 10.8 and 7.0, 8.4 M 41 and 37; folded 4.2 M 60.6
-// and 60.4 (bound by the deposit), 430 K irregular 28 and 19; piecewise linear
+// tracers 9.8 and 6.2, 262 K 10.8 and 7.0, 8.4 M 41 and 37, 430 K irregular 28
+// and 19; folded 4.2 M hardly less (bound by the deposit); piecewise linear
 // 0.5 M 72 and 43, first order 0.5 M 20.7 and 12.5.  What is left of a small
 // step is two trips to L2 (the atomics, the wait) and the scan.
 template <bool PER_Q, bool GEN>
