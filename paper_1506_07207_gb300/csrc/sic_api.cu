@@ -436,21 +436,60 @@ constexpr int kOneBlockItems = 16;
 
 // The groups of blocks of a launch of many steps (k_run), one per simulation:
 // block_begin[slot], and the grid; 0 when the steps are better launched one
-// by one.
-static int split_blocks(sic_sim *const *sims, int n, int nx_max, bool per_q, bool gen, std::vector<int32_t> &block_begin)
+// by one.  Every group gets a block, and the rest go one by one to the
+// simulation with the most work a block: its items, three times as much where
+// the sheets are folded or refined as on quiet ones (a particle that crosses
+// cell edges costs about three that do not; on fresh sheets nx tracers per
+// sheet of them cross, and refined charges mean that the sheets have folded).
+//
+// The gain of such a launch is the fixed cost of a step, 5 to 10 us.  Against
+// it, single simulations lose a little once they stream from HBM (rounds of
+// items, one per warp; us per step, launches of one step and this): 14 rounds
+// 42 and 37, 27 rounds 69 and 69, 55 rounds 112 and 116.  In a batch, blocks
+// do not help another simulation's, so the launch is as slow as the group whose
+// items cost most: 3.4 rounds 24 and 18, 6.7 rounds of 16 simulations 27 and
+// 20, the same half folded 71 and 46, 17 rounds half folded 103 and 115.
+constexpr int kMostRounds = 28;
+constexpr int kMostRoundsBatch = 8;
+
+static int split_blocks(sic_sim *const *sims, int n, int nx_max, int charges, bool gen,
+                        std::vector<int32_t> &block_begin)
 {
-    const int per_sm = run_blocks_per_sm(nx_max, per_q, gen);
-    const int most = env_int("SIC_GRID", num_sms() * per_sm);  // (the test knob of build_plan)
-    if (per_sm < 1 || n != 1)
+    const int per_sm = run_blocks_per_sm(nx_max, charges, gen);
+    // (SIC_GRID: the test knob of build_plan)
+    const int most = std::min(num_sms() * per_sm, std::max(n, env_int("SIC_GRID", num_sms() * per_sm)));
+    if (per_sm < 1 || n > most)
+        return 0;
+    std::vector<int> blocks(n, 1), wanted(n);
+    std::vector<double> work(n);
+    std::vector<std::pair<double, int>> heap;  // work a block, slot
+    for (int i = 0; i < n; ++i) {
+        const sic_sim *m = sims[i];
+        const int items = (int)m->items.size();
+        const double cross = m->seg_q ? 1.0 : std::min(1.0, (double)m->nx * m->M / (double)m->n_tracers);
+        work[i] = items * (1.0 + 2.0 * cross);
+        wanted[i] = items <= kOneBlockItems ? 1 : (items + SIC_K1_WARPS - 1) / SIC_K1_WARPS;
+        if (wanted[i] > 1)
+            heap.emplace_back(work[i], i);
+    }
+    std::make_heap(heap.begin(), heap.end());
+    for (int left = most - n; left > 0 && !heap.empty(); --left) {
+        std::pop_heap(heap.begin(), heap.end());
+        const int i = heap.back().second;
+        heap.pop_back();
+        if (++blocks[i] < wanted[i]) {
+            heap.emplace_back(work[i] / blocks[i], i);
+            std::push_heap(heap.begin(), heap.end());
+        }
+    }
+    int rounds = 0;
+    for (int i = 0; i < n; ++i)
+        rounds = std::max(rounds, ((int)sims[i]->items.size() + SIC_K1_WARPS * blocks[i] - 1) / (SIC_K1_WARPS * blocks[i]));
+    if (rounds > (n == 1 ? kMostRounds : kMostRoundsBatch))
         return 0;
     block_begin.assign(n + 1, 0);
-    for (int slot = 0; slot < n; ++slot) {
-        const int items = (int)sims[slot]->items.size();
-        int blocks = (items + SIC_K1_WARPS - 1) / SIC_K1_WARPS;
-        if (items <= kOneBlockItems)
-            blocks = 1;
-        block_begin[slot + 1] = block_begin[slot] + std::max(1, std::min({blocks, most, num_sms() * per_sm}));
-    }
+    for (int i = 0; i < n; ++i)
+        block_begin[i + 1] = block_begin[i] + blocks[i];
     return block_begin[n];
 }
 
@@ -494,7 +533,9 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     for (int slot = 0; slot < n; ++slot)
         gen = gen || sims[slot]->deposit != SIC_DEPOSIT_BOX;
     std::vector<int32_t> block_begin;
-    p.run_grid = split_blocks(sims, n, nx_max, per_q, gen, block_begin);
+    p.run_grid = n == 1 ? split_blocks(sims, n, nx_max, per_q ? 1 : 0, gen, block_begin) : 0;
+    p.run_charges = per_q ? 1 : 0;
+    p.run_gen = gen;
     Layout lay;
     const size_t oT = lay.take(sizeof(SimDev) * table.size());
     const size_t oS = lay.take(4 * slot_begin.size());
@@ -534,6 +575,45 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     return cudaSuccess;
 }
 
+cudaError_t build_many_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
+{
+    std::vector<SimDev> table(n);
+    int nx_max = 2, per_q = 0;
+    bool gen = false;
+    for (int i = 0; i < n; ++i) {
+        table[i] = sims[i]->h;
+        nx_max = std::max(nx_max, sims[i]->nx);
+        per_q += sims[i]->per_q ? 1 : 0;
+        gen = gen || sims[i]->deposit != SIC_DEPOSIT_BOX;
+    }
+    p.run_charges = per_q == 0 ? 0 : per_q == n ? 1 : 2;
+    p.run_gen = gen;
+    std::vector<int32_t> block_begin;
+    p.run_grid = split_blocks(sims, n, nx_max, p.run_charges, gen, block_begin);
+    if (!p.run_grid)
+        return cudaSuccess;
+    Layout lay;
+    const size_t oT = lay.take(sizeof(SimDev) * table.size());
+    const size_t oB = lay.take(4 * block_begin.size());
+    const size_t oC = lay.take(sizeof(RunCtl) * (size_t)n);
+    cudaError_t e = cudaMallocAsync(&p.mem, lay.off, s);
+    if (e != cudaSuccess) {
+        p.mem = nullptr;
+        p.run_grid = 0;
+        return e;
+    }
+    char *b = (char *)p.mem;
+    e = cudaMemcpyAsync(b + oT, table.data(), sizeof(SimDev) * table.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b + oB, block_begin.data(), 4 * block_begin.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(b + oC, 0, sizeof(RunCtl) * (size_t)n, s);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(s);  // host staging vectors go out of scope
+    p.run = RunArgs{(const SimDev *)(b + oT), (const int32_t *)(b + oB), (RunCtl *)(b + oC), n, nx_max, 0};
+    return e;
+}
+
 void set_schedule(Plan &p, int claim_div, int staging, int claim_min)
 {
     p.args.claim_q = (float)(1.0 / ((double)std::max(1, claim_div) * p.grid * SIC_K1_WARPS));
@@ -546,7 +626,7 @@ constexpr int kStepsALaunch = 256;
 bool launch_many(Plan &p, int n_steps, cudaStream_t s, cudaError_t &e)
 {
     e = cudaSuccess;
-    if (!p.run_grid || n_steps < 2)
+    if (!p.run_grid || n_steps < (p.args.n_slots ? 2 : 1))  // (a single step is as well launched by itself)
         return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
@@ -554,7 +634,7 @@ bool launch_many(Plan &p, int n_steps, cudaStream_t s, cudaError_t &e)
     for (int left = n_steps; left > 0 && e == cudaSuccess;) {
         RunArgs a = p.run;
         a.n_steps = std::min(left, kStepsALaunch);
-        e = launch_run_kernel(a, p.run_grid, p.per_q, p.args.gen != 0, s);
+        e = launch_run_kernel(a, p.run_grid, p.run_charges, p.run_gen, s);
         if (left == n_steps && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
             cudaGetLastError();  // not on this device: one launch a step from now on
             e = cudaSuccess;
@@ -1162,6 +1242,21 @@ int sic_step_batch(sic_sim *const *sims, int32_t n_sims, const int32_t *n_steps)
         if (grp[0].empty() && grp[1].empty())
             break;
         Plan plans[2];
+        {
+            std::vector<sic_sim *> both(grp[0]);
+            both.insert(both.end(), grp[1].begin(), grp[1].end());
+            Plan many;
+            cudaError_t e = build_many_plan(many, both.data(), (int)both.size(), bs);
+            const bool ran = e == cudaSuccess && launch_many(many, k, bs, e);
+            free_plan(many, bs);
+            CK(e);
+            if (ran) {
+                for (int i = 0; i < n_sims; ++i)
+                    if (left[i] > 0)
+                        left[i] -= k;
+                continue;
+            }
+        }
         for (int g = 0; g < 2; ++g)
             if (!grp[g].empty())
                 CK(build_plan(plans[g], grp[g].data(), (int)grp[g].size(), bs));
@@ -1192,6 +1287,7 @@ struct sic_batch {
     std::vector<sic_sim *> sims;
     cudaStream_t stream = nullptr;
     sic_host::Plan plan[2];
+    sic_host::Plan many;  // all members, many steps a launch (when it is taken)
     cudaGraphExec_t gexec = nullptr;
     int64_t segments = 0;
 };
@@ -1254,6 +1350,13 @@ int sic_batch_create(sic_sim *const *sims, int32_t n_sims, sic_batch **out)
                 return e == cudaErrorMemoryAllocation ? SIC_ENOMEM : SIC_ECUDA;
             }
         }
+    {
+        const cudaError_t e = sic_host::build_many_plan(b->many, b->sims.data(), n_sims, b->stream);
+        if (e != cudaSuccess) {
+            sic_batch_destroy(b);
+            return e == cudaErrorMemoryAllocation ? SIC_ENOMEM : SIC_ECUDA;
+        }
+    }
     *out = b;
     return SIC_OK;
 }
@@ -1263,6 +1366,11 @@ int sic_batch_step(sic_batch *b, int32_t n_steps)
     if (!b || n_steps < 0)
         return SIC_EINVAL;
     sic_sim *sim = b->sims[0];
+    {
+        cudaError_t e;
+        if (sic_host::launch_many(b->many, n_steps, b->stream, e))
+            return e == cudaSuccess ? SIC_OK : fail_cuda(sim, e);
+    }
     const int launches_per_step = (b->plan[0].mem ? 1 : 0) + (b->plan[1].mem ? 1 : 0);
     if (n_steps >= kGraphSteps && !b->gexec) {
         cudaGraph_t g = nullptr;
@@ -1360,6 +1468,7 @@ void sic_batch_destroy(sic_batch *b)
         cudaGraphExecDestroy(b->gexec);
     for (auto &p : b->plan)
         sic_host::free_plan(p, b->stream);
+    sic_host::free_plan(b->many, b->stream);
     cudaEvent_t done;
     if (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess) {
         cudaEventRecord(done, b->stream);

@@ -20,6 +20,8 @@ struct Plan {
     bool per_q = false;
     RunArgs run{};       // many steps in one launch (run_grid 0: not for this plan)
     int run_grid = 0;
+    int run_charges = 0;
+    bool run_gen = false;
 };
 
 // Device bytes of one simulation's allocation (state, meshes, items, ...).
@@ -82,6 +84,11 @@ int refine_held(sic_sim *sim, int64_t *added);
 // Particles (segments) of the simulation now.
 int64_t segments(const sic_sim *sim);
 cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s);
+// The plan of launches of many steps over simulations of either charge mode
+// (launch_many alone takes it): run_grid stays 0, and nothing is allocated,
+// where such launches do not fit or the simulations are better balanced in
+// launches of one step.
+cudaError_t build_many_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s);
 // Scheduling knobs of a built plan (results do not depend on them): the claim
 // divisor D (a claim takes 1 / (D warps) of what is left) and the staging
 // choice (LaunchArgs::staging).

@@ -180,13 +180,16 @@ struct LaunchArgs {
 };
 
 // What the blocks of one simulation share in a launch of k_run (all zero
-// between launches): the sums of three steps (SimAccum::pad[0]: error bits)
-// and the counts of blocks that have finished a step and that have left.
+// between launches): the sums of three steps (SimAccum::pad[0]: error bits),
+// their claims of items, and the counts of blocks that have finished a step
+// and that have left.
 struct RunCtl {
     SimAccum acc[3];
     unsigned bar;
+    unsigned pad0[31];
+    unsigned cursor[3];
     unsigned out;
-    unsigned pad[30];
+    unsigned pad1[28];
 };
 
 // One launch of k_run: n_steps steps of every simulation.
@@ -205,8 +208,9 @@ enum Mode { MODE_STEP = 0, MODE_DEPOSIT = 1, MODE_PUSH = 2 };
 cudaError_t launch_step_kernel(const LaunchArgs &a, int grid, Mode mode, bool per_q, cudaStream_t s);
 // Many steps in one cooperative launch; the blocks of it an SM holds (0: the
 // meshes are too large for it)
-cudaError_t launch_run_kernel(const RunArgs &a, int grid, bool per_q, bool gen, cudaStream_t s);
-int run_blocks_per_sm(int nx_max, bool per_q, bool gen);
+// charges: 0 one per sheet in every simulation, 1 per tracer in every one, 2 either
+cudaError_t launch_run_kernel(const RunArgs &a, int grid, int charges, bool gen, cudaStream_t s);
+int run_blocks_per_sm(int nx_max, int charges, bool gen);
 cudaError_t launch_field_out(const SimDev &sim, cudaStream_t s);
 cudaError_t launch_spectrum(const SimDev &sim, int field, cudaStream_t s);
 cudaError_t launch_refine_count(const SimDev &sim, long long lfix, int32_t *splits, cudaStream_t s);

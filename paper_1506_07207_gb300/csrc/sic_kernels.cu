@@ -2155,7 +2155,7 @@ __device__ __forceinline__ bool group_wait(const unsigned *bar, unsigned target)
 // 0.5 M 72 and 43, first order 0.5 M 20.7 and 12.5.  What is left of a small
 // step is two trips to L2 (the atomics, the wait) and the scan.
 template <bool PER_Q, bool GEN>
-__global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
+__device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     Shared &sh = *reinterpret_cast<Shared *>(smem);
@@ -2174,17 +2174,6 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
     unsigned short *tasks =
         reinterpret_cast<unsigned short *>(stage_base + (size_t)NW * WarpBuf<PER_Q, true>::bytes) + warp * WT;
 
-    int slot = 0;
-    {
-        int hi = A.n_slots - 1;  // the last slot whose blocks begin at or before this one
-        while (slot < hi) {
-            const int mid = (slot + hi + 1) >> 1;
-            if (A.block_begin[mid] <= (int)blockIdx.x)
-                slot = mid;
-            else
-                hi = mid - 1;
-        }
-    }
     const int rank = (int)blockIdx.x - A.block_begin[slot];
     const int G = A.block_begin[slot + 1] - A.block_begin[slot];
     const bool recorder = rank == G - 1;
@@ -2233,6 +2222,13 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
     const bool track_all = S.refine_seg > 0 && S.refine_seg < (1ll << 16);  // refinement below a cell
     const int32_t *Qh = S.Qh;
     const int stride = G * NW, first = warp * G + rank;
+    // The first three quarters of the rounds are the warp's own items (first,
+    // first + stride, ...); the rest are claimed one at a time, an item ahead,
+    // since folded and quiet sheets differ by a factor of three.
+    const int rounds = (n_items + stride - 1) / stride;
+    const bool claims = G > 1 && rounds > 1;
+    const int own = claims ? max(1, rounds * 3 / 4) : rounds;
+    unsigned claimed = 0;  // lane 0: the claim in flight
 
     unsigned phase = 0;
     int s = 0;
@@ -2243,8 +2239,11 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
         stage_issue<PER_Q>(sh.desc[warp][stage].w, S.U[from], S.V[from], Qh, my_stage + stage * WarpBuf<PER_Q, true>::stage,
                            &sh.mbar[warp][stage]);
     };
-    if (first < n_items && lane == 0)
+    if (first < n_items && lane == 0) {
         issue(first, s, src);
+        if (claims && own == 1)
+            claimed = atomicAdd(&ctl->cursor[0], 1u);
+    }
     __syncwarp();
 
     for (int st = 0;; ++st) {
@@ -2258,6 +2257,8 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
                 m[j] = 0ull;
             if (tid < (int)(sizeof(SimAccum) / 8))
                 reinterpret_cast<unsigned long long *>(&ctl->acc[nxt_buf])[tid] = 0ull;
+            if (tid == 32)
+                ctl->cursor[nxt_buf] = 0u;
         }
         // ---- 1. items
         const unsigned *Uin = S.U[src];
@@ -2266,8 +2267,17 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
         float *Vout = S.V[src ^ 1];
         unsigned rerr = 0, mseg = 0, mlen = 0;
         long long ake = 0, ap = 0;
-        for (int i = first; i < n_items; i += stride) {
-            const int nxt = i + stride < n_items ? i + stride : -1;
+        for (int i = first, r = 0; i >= 0 && i < n_items; ++r) {
+            int nxt;
+            if (r + 1 < own)
+                nxt = i + stride;
+            else if (claims)
+                nxt = own * stride + (int)__shfl_sync(0xffffffffu, claimed, 0);
+            else
+                nxt = n_items;
+            nxt = nxt < n_items ? nxt : -1;
+            if (claims && r + 2 >= own && nxt >= 0 && lane == 0)
+                claimed = atomicAdd(&ctl->cursor[now], 1u);
             const WorkItem W = sh.desc[warp][s].w;
             const WorkItemPL *plw = (GEN && S.pl != nullptr) ? S.pl + i : nullptr;
             if (nxt >= 0 && lane == 0)
@@ -2298,6 +2308,7 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
                                                             S.seg_q, track_all, mid);
             __syncwarp();
             s ^= 1;
+            i = nxt;
         }
 
         // ---- 2. the block's mesh and sums
@@ -2410,6 +2421,8 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
         if (!last && first < n_items && lane == 0) {
             asm volatile("fence.proxy.async;" ::: "memory");
             issue(first, s, src);
+            if (claims && own == 1)
+                claimed = atomicAdd(&ctl->cursor[nxt_buf], 1u);
         }
         if (last && !recorder)
             break;
@@ -2593,6 +2606,8 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
             S.mesh[j] = 0ull;
         for (int i = tid; i < (int)(sizeof(ctl->acc) / 8); i += B)
             reinterpret_cast<unsigned long long *>(ctl->acc)[i] = 0ull;
+        if (tid < 3)
+            ctl->cursor[tid] = 0u;
     }
     if (tid == 0 && atomicAdd(&ctl->out, 1u) + 1 == (unsigned)G) {
         ctl->out = 0u;
@@ -2600,7 +2615,34 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
     }
 }
 
-template <bool Q, bool G>
+// The slot whose group this block belongs to: the last one whose blocks begin
+// at or before it
+__device__ __forceinline__ int run_slot(const RunArgs &A)
+{
+    int slot = 0, hi = A.n_slots - 1;
+    while (slot < hi) {
+        const int mid = (slot + hi + 1) >> 1;
+        if (A.block_begin[mid] <= (int)blockIdx.x)
+            slot = mid;
+        else
+            hi = mid - 1;
+    }
+    return slot;
+}
+
+// Charges: 0 one per sheet in every simulation, 1 per tracer in every one, 2
+// either (a block's simulation decides)
+template <int CHARGES, bool GEN>
+__global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
+{
+    const int slot = run_slot(A);
+    if (CHARGES == 1 || (CHARGES == 2 && A.sims[slot].Qh != nullptr))
+        run_steps<true, GEN>(A, slot);
+    else
+        run_steps<false, GEN>(A, slot);
+}
+
+template <int Q, bool G>
 cudaError_t prep_run(size_t smem)
 {
     static size_t done = 0;
@@ -2614,10 +2656,10 @@ cudaError_t prep_run(size_t smem)
     return cudaSuccess;
 }
 
-template <bool Q, bool G>
+template <int Q, bool G>
 cudaError_t run_many(const RunArgs &a, int grid, cudaStream_t s)
 {
-    const size_t smem = step_smem_bytes(a.nx_max, true, Q);
+    const size_t smem = step_smem_bytes(a.nx_max, true, Q != 0);
     cudaError_t e = prep_run<Q, G>(smem);
     if (e != cudaSuccess)
         return e;
@@ -2637,10 +2679,10 @@ cudaError_t run_many(const RunArgs &a, int grid, cudaStream_t s)
     return e;
 }
 
-template <bool Q, bool G>
+template <int Q, bool G>
 int occ_run(int nx_max)
 {
-    const size_t smem = step_smem_bytes(nx_max, true, Q);
+    const size_t smem = step_smem_bytes(nx_max, true, Q != 0);
     if (smem > 227 * 1024 || prep_run<Q, G>(smem) != cudaSuccess)
         return 0;
     int n = 0;
@@ -2901,18 +2943,22 @@ int step_blocks_per_sm(int nx_max, Mode mode, bool per_q)
     }
 }
 
-cudaError_t launch_run_kernel(const RunArgs &a, int grid, bool per_q, bool gen, cudaStream_t s)
+cudaError_t launch_run_kernel(const RunArgs &a, int grid, int charges, bool gen, cudaStream_t s)
 {
-    if (gen)
-        return per_q ? run_many<true, true>(a, grid, s) : run_many<false, true>(a, grid, s);
-    return per_q ? run_many<true, false>(a, grid, s) : run_many<false, false>(a, grid, s);
+    if (charges == 0)
+        return gen ? run_many<0, true>(a, grid, s) : run_many<0, false>(a, grid, s);
+    if (charges == 1)
+        return gen ? run_many<1, true>(a, grid, s) : run_many<1, false>(a, grid, s);
+    return gen ? run_many<2, true>(a, grid, s) : run_many<2, false>(a, grid, s);
 }
 
-int run_blocks_per_sm(int nx_max, bool per_q, bool gen)
+int run_blocks_per_sm(int nx_max, int charges, bool gen)
 {
-    if (gen)
-        return per_q ? occ_run<true, true>(nx_max) : occ_run<false, true>(nx_max);
-    return per_q ? occ_run<true, false>(nx_max) : occ_run<false, false>(nx_max);
+    if (charges == 0)
+        return gen ? occ_run<0, true>(nx_max) : occ_run<0, false>(nx_max);
+    if (charges == 1)
+        return gen ? occ_run<1, true>(nx_max) : occ_run<1, false>(nx_max);
+    return gen ? occ_run<2, true>(nx_max) : occ_run<2, false>(nx_max);
 }
 
 cudaError_t launch_field_out(const SimDev &sim, cudaStream_t s)

@@ -74,6 +74,7 @@ struct sic_server {
     int64_t next_id = 1;
     size_t used = 0, peak = 0;
     sic_host::Plan plan[2];
+    sic_host::Plan many;                    // all active ones, many steps a launch (when it is taken)
     bool plan_valid = false;
     Clock::time_point t0;
     int64_t completed = 0, segment_updates = 0, ticks = 0;
@@ -92,6 +93,8 @@ void drop_plans(sic_server *s)
 {
     for (auto &p : s->plan)
         sic_host::free_plan(p, s->stream);
+    sic_host::free_plan(s->many, s->stream);
+    s->many.run_grid = 0;
     s->plan_valid = false;
 }
 
@@ -341,10 +344,14 @@ int tick_batched(sic_server *srv)
         int lrc = SIC_OK;
         if (k > 0 && !srv->plan_valid) {
             drop_plans(srv);
-            std::vector<sic_sim *> grp[2];
-            for (const Active &a : srv->active)
+            std::vector<sic_sim *> all, grp[2];
+            for (const Active &a : srv->active) {
+                all.push_back(a.sim);
                 grp[a.sim->per_q ? 1 : 0].push_back(a.sim);
-            for (int g = 0; g < 2 && lrc == SIC_OK; ++g)
+            }
+            if (sic_host::build_many_plan(srv->many, all.data(), (int)all.size(), srv->stream) != cudaSuccess)
+                lrc = SIC_ECUDA;
+            for (int g = 0; g < 2 && lrc == SIC_OK && !srv->many.run_grid; ++g)
                 if (!grp[g].empty() &&
                     sic_host::build_plan(srv->plan[g], grp[g].data(), (int)grp[g].size(), srv->stream) != cudaSuccess)
                     lrc = SIC_ECUDA;
@@ -357,7 +364,21 @@ int tick_batched(sic_server *srv)
             cudaEventRecord(srv->ev[1], srv->stream);
         } else if (k > 0) {
             cudaEventRecord(srv->ev[0], srv->stream);
-            for (int32_t st = 0; st < k && lrc == SIC_OK; ++st)
+            cudaError_t e = cudaSuccess;
+            const bool ran = sic_host::launch_many(srv->many, k, srv->stream, e);
+            if (e != cudaSuccess)
+                lrc = SIC_ECUDA;
+            if (!ran && lrc == SIC_OK && !srv->plan[0].mem && !srv->plan[1].mem) {
+                // the device does not take such launches after all
+                std::vector<sic_sim *> grp[2];
+                for (const Active &a : srv->active)
+                    grp[a.sim->per_q ? 1 : 0].push_back(a.sim);
+                for (int g = 0; g < 2 && lrc == SIC_OK; ++g)
+                    if (!grp[g].empty() && sic_host::build_plan(srv->plan[g], grp[g].data(), (int)grp[g].size(),
+                                                                srv->stream) != cudaSuccess)
+                        lrc = SIC_ECUDA;
+            }
+            for (int32_t st = 0; !ran && st < k && lrc == SIC_OK; ++st)
                 for (int g = 0; g < 2 && lrc == SIC_OK; ++g)
                     if (srv->plan[g].mem &&
                         sic_host::launch(srv->plan[g], sic::MODE_STEP, 1.0f, 1, 1, srv->stream) != cudaSuccess)
