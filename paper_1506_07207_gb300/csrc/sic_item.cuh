@@ -461,16 +461,18 @@ __device__ __forceinline__ void acc_add(Acc128 &a, const Acc128 &b)
     a.lo = nlo;
 }
 
-__device__ __forceinline__ Acc128 acc_warp_sum(Acc128 a)
+// The sum of the warp's 64-bit values, in every lane: four sums of 16-bit
+// pieces (the top one signed), 21 bits each, by the warp's own reduction
+__device__ __forceinline__ Acc128 i64_warp_sum(long long v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Acc128 t;
-        t.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
-        t.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
-        acc_add(a, t);
-    }
-    return a;
+    const unsigned long long u = (unsigned long long)v;
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)u & 0xffffu);
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 16) & 0xffffu);
+    const unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 32) & 0xffffu);
+    const int s3 = __reduce_add_sync(0xffffffffu, (int)(v >> 48));
+    Acc128 t{(unsigned long long)s0 + ((unsigned long long)s1 << 16) + ((unsigned long long)s2 << 32), 0ll};
+    acc_add(t, Acc128{(unsigned long long)(long long)s3 << 48, (long long)s3 >> 16});
+    return t;
 }
 
 // 128-bit add into a (lo, hi) pair of 64-bit words with two atomics
@@ -662,6 +664,16 @@ __device__ __forceinline__ void stage_issue(const WorkItem &W, const unsigned *U
         bulk_g2s(st + kStageBytesU + kStageBytesV, Qh + W.t0, b, bar, pol);
 }
 
+// What a warp that keeps its item in shared memory from step to step (k_run)
+// holds besides: the tracers outside the item that it pushes for itself, the
+// one after the item and, for piecewise-linear particles, the one before it
+// and the one after the next
+struct Beside {
+    unsigned hu, pu, nu;
+    float hv, pv, nv;
+    int hq, pq, nq;
+};
+
 struct Shared {
     SimDev sim;              // the current simulation's descriptor
     unsigned long long mbar[NW][2];
@@ -693,6 +705,8 @@ struct Shared {
     unsigned long long step_mseg;
     unsigned step_err, gave_up;
     unsigned long long tot[2][2];  // KE, P: lo, hi
+    WorkItem own[NW];              // each warp's first item of a step
+    Beside beside[NW];
 };
 
 constexpr size_t kSharedHead = (sizeof(Shared) + 15) / 16 * 16;
@@ -751,9 +765,15 @@ __device__ __forceinline__ Norm128 norm128(__int128 v)
     r.neg = v < 0;
     const unsigned __int128 m = r.neg ? (unsigned __int128)(-v) : (unsigned __int128)v;
     const unsigned long long hi = (unsigned long long)(m >> 64), lo = (unsigned long long)m;
-    const int lz = hi ? __clzll((long long)hi) : (lo ? 64 + __clzll((long long)lo) : 0);
-    r.t = (unsigned)((m << lz) >> 96);
-    r.e = 96 - lz;
+    // the top two nonzero 32-bit words and a funnel shift, instead of a
+    // 128-bit one
+    const unsigned long long top = hi ? hi : lo;
+    const unsigned th = (unsigned)(top >> 32), tl = (unsigned)top;
+    const unsigned a = th ? th : tl;
+    const unsigned b = th ? tl : (hi ? (unsigned)(lo >> 32) : 0u);
+    const int lz = __clz((int)a);
+    r.t = __funnelshift_l(b, a, lz);
+    r.e = (hi ? 64 : 0) + (th ? 32 : 0) - lz;
     return r;
 }
 
@@ -763,8 +783,13 @@ __device__ __forceinline__ float norm_to_float(const Norm128 &n, int e2)
     if (n.zero)
         return 0.f;
     const int e = n.e + e2;  // |v| 2^e2 = t 2^e
-    const int e_a = e / 2, e_b = e - e / 2;
-    const float f = __fmul_rn(__fmul_rn(__uint2float_rn(n.t), pow2f(e_a)), pow2f(e_b));
+    float f = __uint2float_rn(n.t);
+    if (e >= -126 && e <= 95) {  // one exact scaling
+        f = __fmul_rn(f, __uint_as_float((unsigned)(e + 127) << 23));
+    } else {
+        const int e_a = e / 2, e_b = e - e / 2;
+        f = __fmul_rn(__fmul_rn(f, pow2f(e_a)), pow2f(e_b));
+    }
     return n.neg ? -f : f;
 }
 
@@ -970,14 +995,17 @@ __device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int 
 }
 
 // One work item (up to 32 R tracers, R per lane) of the current simulation.
-// FULL: the item has all 32 R tracers, so no lane needs a bounds test.
-template <bool PUSH, bool DEPOSIT, bool PER_Q, bool FULL, bool STAGED, bool GEN, class MID>
+// FULL: the item has all 32 R tracers, so no lane needs a bounds test.  KEPT:
+// the item stays in its stage st from step to step (k_run): it is written back
+// there, and the tracers beside it are kept in sh.beside; tab is then a table
+// of its own.
+template <bool PUSH, bool DEPOSIT, bool PER_Q, bool FULL, bool STAGED, bool GEN, bool KEPT, class MID>
 __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__restrict__ Uin,
                                         const float *__restrict__ Vin, unsigned *__restrict__ Uout,
                                         float *__restrict__ Vout, const int32_t *__restrict__ Qh,
                                         const float2 *ek, const Hist &hist, const Hist &diff,
                                         Shared &sh, int nx, float ks, int drift, unsigned &rerr,
-                                        char *st, unsigned short *tasks, long long &ake, long long &ap, unsigned &mseg, unsigned &mlen,
+                                        char *st, char *tab, unsigned short *tasks, long long &ake, long long &ap, unsigned &mseg, unsigned &mlen,
                                         const WorkItemPL *pw, int dep, int segq, bool track_all, const MID &mid)
 {
     const unsigned *stU = reinterpret_cast<const unsigned *>(st);
@@ -1007,9 +1035,15 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
     float hv = 0.f;
     int hq = W.qh, hj = 0;
     bool has_halo = false;
+    Beside &beside = sh.beside[threadIdx.x >> 5];
     if (DEPOSIT && lane == lane_last && W.halo >= 0) {
         has_halo = true;
-        if (STAGED && W.halo == base + m) {
+        if (KEPT) {
+            hu = beside.hu;
+            hv = beside.hv;
+            if (PER_Q)
+                hq = beside.hq;
+        } else if (STAGED && W.halo == base + m) {
             hu = stU[m];
             if (PUSH)
                 hv = stV[m];
@@ -1091,8 +1125,21 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
         if (has_halo) {
             float ignore = 0.f;
             push_one(hu, hv, hj, ek, nx, ks, drift, ignore);
+            if (KEPT) {
+                beside.hu = hu;
+                beside.hv = hv;
+            }
         }
-        if (FULL || rn == R) {
+        if (KEPT) {
+            // back to the stage (past the item's end: what was there)
+            unsigned *bu = reinterpret_cast<unsigned *>(st) + l0;
+            float *bv = reinterpret_cast<float *>(st + kStageBytesU) + l0;
+#pragma unroll
+            for (int k = 0; k < R / 4; ++k) {
+                reinterpret_cast<uint4 *>(bu)[k] = make_uint4(u[4 * k], u[4 * k + 1], u[4 * k + 2], u[4 * k + 3]);
+                reinterpret_cast<float4 *>(bv)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            }
+        } else if (FULL || rn == R) {
 #pragma unroll
             for (int k = 0; k < R / 4; ++k) {
                 __stcs(reinterpret_cast<uint4 *>(Uout + base + l0) + k,
@@ -1130,26 +1177,34 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
         has_prev = ip >= 0;
         has_next2 = in2 >= 0;
         if (lane == 0 && has_prev) {
-            pu = __ldcg(Uin + ip);
+            pu = KEPT ? beside.pu : __ldcg(Uin + ip);
             if (PER_Q)
-                pq = Qh[ip];
+                pq = KEPT ? beside.pq : Qh[ip];
             if (PUSH) {
-                float pv = __ldcg(Vin + ip);
+                float pv = KEPT ? beside.pv : __ldcg(Vin + ip);
                 int pj;
                 float ignore = 0.f;
                 push_one(pu, pv, pj, ek, nx, ks, drift, ignore);
+                if (KEPT) {
+                    beside.pu = pu;
+                    beside.pv = pv;
+                }
             }
             pu -= pw->prev_shift;
         }
         if (lane == lane_last && has_next2) {
-            nu2 = __ldcg(Uin + in2);
+            nu2 = KEPT ? beside.nu : __ldcg(Uin + in2);
             if (PER_Q)
-                nq2 = Qh[in2];
+                nq2 = KEPT ? beside.nq : Qh[in2];
             if (PUSH) {
-                float nv = __ldcg(Vin + in2);
+                float nv = KEPT ? beside.nv : __ldcg(Vin + in2);
                 int nj;
                 float ignore = 0.f;
                 push_one(nu2, nv, nj, ek, nx, ks, drift, ignore);
+                if (KEPT) {
+                    beside.nu = nu2;
+                    beside.nv = nv;
+                }
             }
             nu2 += pw->next2_shift;
         }
@@ -1196,7 +1251,7 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
                 --nseg;
         }
         deposit_boxes<PER_Q, FULL>(u, jn, q, nu, nj, nq, nseg, rn, m - (W.halo >= 0 ? 0 : 1), 2 * W.qh, segq, nx,
-                                   hist, diff, &sh.diff_used, reinterpret_cast<unsigned *>(st), mlen);
+                                   hist, diff, &sh.diff_used, reinterpret_cast<unsigned *>(tab), mlen);
         if (track_all) {
             // a refinement length shorter than a cell: particles inside one
             // cell count towards the longest one too

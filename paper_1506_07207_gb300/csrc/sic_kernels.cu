@@ -442,24 +442,24 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
                     };
                     char *st = my_stage + s * WarpBuf<PER_Q, true>::stage;
                     if (W.count == WT)
-                        do_item<PUSH, DEPOSIT, PER_Q, true, true, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                  nx, ks, drift, rerr, st, tasks, ake, ap, mseg, mlen, plw,
+                        do_item<PUSH, DEPOSIT, PER_Q, true, true, GEN, false>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
+                                                                  nx, ks, drift, rerr, st, st, tasks, ake, ap, mseg, mlen, plw,
                                                                   S.deposit, S.seg_q, track_all, mid);
                     else
-                        do_item<PUSH, DEPOSIT, PER_Q, false, true, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                   nx, ks, drift, rerr, st, tasks, ake, ap, mseg, mlen, plw,
+                        do_item<PUSH, DEPOSIT, PER_Q, false, true, GEN, false>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
+                                                                   nx, ks, drift, rerr, st, st, tasks, ake, ap, mseg, mlen, plw,
                                                                    S.deposit, S.seg_q, track_all, mid);
                     __syncwarp();
                     s ^= 1;
                 } else {
                     auto mid = []() {};
                     if (W.count == WT)
-                        do_item<PUSH, DEPOSIT, PER_Q, true, false, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                   nx, ks, drift, rerr, my_stage, tasks, ake, ap, mseg, mlen,
+                        do_item<PUSH, DEPOSIT, PER_Q, true, false, GEN, false>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
+                                                                   nx, ks, drift, rerr, my_stage, my_stage, tasks, ake, ap, mseg, mlen,
                                                                    plw, S.deposit, S.seg_q, track_all, mid);
                     else
-                        do_item<PUSH, DEPOSIT, PER_Q, false, false, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
-                                                                    nx, ks, drift, rerr, my_stage, tasks, ake, ap, mseg, mlen,
+                        do_item<PUSH, DEPOSIT, PER_Q, false, false, GEN, false>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh,
+                                                                    nx, ks, drift, rerr, my_stage, my_stage, tasks, ake, ap, mseg, mlen,
                                                                     plw, S.deposit, S.seg_q, track_all, mid);
                 }
             }
@@ -482,8 +482,8 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
         // ---- leave: fold the block's mesh and sums into the simulation's,
         // take an item ticket, run the field epilogue if it completes it
         if (PUSH) {
-            const Acc128 k2 = acc_warp_sum(Acc128{(unsigned long long)ake, ake >> 63});
-            const Acc128 p2 = acc_warp_sum(Acc128{(unsigned long long)ap, ap >> 63});
+            const Acc128 k2 = i64_warp_sum(ake);
+            const Acc128 p2 = i64_warp_sum(ap);
             if (lane == 0) {
                 sh.wke[warp][0] = (long long)k2.lo;
                 sh.wke[warp][1] = k2.hi;

@@ -42,10 +42,13 @@ __device__ __forceinline__ bool group_wait(const unsigned *bar, unsigned target)
 // k_field_out writes on request, serve as the second and third mesh.
 //
 // us per step in runs of 160 steps, graphs of single steps and this: 4 K
-// tracers 9.8 and 6.2, 262 K 10.8 and 7.0, 8.4 M 41 and 37, 430 K irregular 28
-// and 19; folded 4.2 M hardly less (bound by the deposit); piecewise linear
-// 0.5 M 72 and 43, first order 0.5 M 20.7 and 12.5.  What is left of a small
-// step is two trips to L2 (the atomics, the wait) and the scan.
+// tracers 9.8 and 6.3, 262 K 10.8 and 5.7, 430 K irregular 28 and 16, 8.4 M 41
+// and 36; piecewise linear 0.5 M 72 and 42, first order 0.5 M 20.7 and 10.3.
+// Folded 2.3 M and 4.2 M go from 33.8 to 32.1 and from 50.6 to 46.1 (bound by
+// the deposit).  Up to one item a warp (622 K tracers) the tracers never leave
+// shared memory between the first step and the last: with their copies 262 K
+// took 7.1, first order 12.6.  What is left of a small step (262 K: about 2 us
+// the items, 3 the adds into L2 and the wait, 1.5 the field) are latencies.
 template <bool PER_Q, bool GEN>
 __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
 {
@@ -125,18 +128,46 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
     unsigned phase = 0;
     int s = 0;
     bool timed_out = false;
-    auto issue = [&](int item, int stage, int from) {  // lane 0: an item's descriptor and copies, from the start
-        desc_fetch(&sh.desc[warp][stage].w, items + item);
+    // A simulation of at most one item a warp is kept: the items stay in their
+    // stages from the first step to the last, which writes them back in place.
+    const bool kept = rounds == 1;
+    const bool busy = first < n_items;
+    if (busy && lane == 0) {
+        desc_fetch(&sh.own[warp], items + first);
         desc_wait();
-        stage_issue<PER_Q>(sh.desc[warp][stage].w, S.U[from], S.V[from], Qh, my_stage + stage * WarpBuf<PER_Q, true>::stage,
-                           &sh.mbar[warp][stage]);
-    };
-    if (first < n_items && lane == 0) {
-        issue(first, s, src);
+        stage_issue<PER_Q>(sh.own[warp], S.U[src], S.V[src], Qh, my_stage, &sh.mbar[warp][0]);
         if (claims && own == 1)
             claimed = atomicAdd(&ctl->cursor[0], 1u);
     }
     __syncwarp();
+    if (kept && busy) {
+        const WorkItem W = sh.own[warp];
+        Beside &b = sh.beside[warp];
+        if (lane == 0 && W.halo >= 0) {
+            b.hu = __ldcg(S.U[src] + W.halo);
+            b.hv = __ldcg(S.V[src] + W.halo);
+            if (PER_Q)
+                b.hq = Qh[W.halo];
+        }
+        if (GEN && S.pl != nullptr && lane == 1) {
+            const WorkItemPL P = S.pl[first];
+            if (P.prev >= 0) {
+                b.pu = __ldcg(S.U[src] + P.prev);
+                b.pv = __ldcg(S.V[src] + P.prev);
+                if (PER_Q)
+                    b.pq = Qh[P.prev];
+            }
+            if (P.next2 >= 0) {
+                b.nu = __ldcg(S.U[src] + P.next2);
+                b.nv = __ldcg(S.V[src] + P.next2);
+                if (PER_Q)
+                    b.nq = Qh[P.next2];
+            }
+        }
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sh.mbar[warp][0], 0u)))
+            timed_out = true;
+        __syncwarp();
+    }
 
     for (int st = 0;; ++st) {
         const int now = st % 3, nxt_buf = (st + 1) % 3;
@@ -159,7 +190,21 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
         float *Vout = S.V[src ^ 1];
         unsigned rerr = 0, mseg = 0, mlen = 0;
         long long ake = 0, ap = 0;
-        for (int i = first, r = 0; i >= 0 && i < n_items; ++r) {
+        if (kept && busy && !timed_out) {
+            const WorkItem W = sh.own[warp];
+            const WorkItemPL *plw = (GEN && S.pl != nullptr) ? S.pl + first : nullptr;
+            char *tab = my_stage + WarpBuf<PER_Q, true>::stage;
+            auto mid = []() {};
+            if (W.count == WT)
+                do_item<true, true, PER_Q, true, true, GEN, true>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh, nx, 1.0f, 1,
+                                                                 rerr, my_stage, tab, tasks, ake, ap, mseg, mlen, plw,
+                                                                 S.deposit, S.seg_q, track_all, mid);
+            else
+                do_item<true, true, PER_Q, false, true, GEN, true>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh, nx, 1.0f,
+                                                                  1, rerr, my_stage, tab, tasks, ake, ap, mseg, mlen, plw,
+                                                                  S.deposit, S.seg_q, track_all, mid);
+        }
+        for (int i = kept ? -1 : first, r = 0; i >= 0 && i < n_items; ++r) {
             int nxt;
             if (r + 1 < own)
                 nxt = i + stride;
@@ -170,7 +215,7 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
             nxt = nxt < n_items ? nxt : -1;
             if (claims && r + 2 >= own && nxt >= 0 && lane == 0)
                 claimed = atomicAdd(&ctl->cursor[now], 1u);
-            const WorkItem W = sh.desc[warp][s].w;
+            const WorkItem W = r == 0 ? sh.own[warp] : sh.desc[warp][s].w;
             const WorkItemPL *plw = (GEN && S.pl != nullptr) ? S.pl + i : nullptr;
             if (nxt >= 0 && lane == 0)
                 desc_fetch(&sh.desc[warp][s ^ 1].w, items + nxt);
@@ -191,12 +236,12 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
             };
             char *stg = my_stage + s * WarpBuf<PER_Q, true>::stage;
             if (W.count == WT)
-                do_item<true, true, PER_Q, true, true, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh, nx, 1.0f, 1,
-                                                           rerr, stg, tasks, ake, ap, mseg, mlen, plw, S.deposit, S.seg_q,
+                do_item<true, true, PER_Q, true, true, GEN, false>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh, nx, 1.0f, 1,
+                                                           rerr, stg, stg, tasks, ake, ap, mseg, mlen, plw, S.deposit, S.seg_q,
                                                            track_all, mid);
             else
-                do_item<true, true, PER_Q, false, true, GEN>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh, nx, 1.0f, 1,
-                                                            rerr, stg, tasks, ake, ap, mseg, mlen, plw, S.deposit,
+                do_item<true, true, PER_Q, false, true, GEN, false>(W, Uin, Vin, Uout, Vout, Qh, ek, hist, diff, sh, nx, 1.0f, 1,
+                                                            rerr, stg, stg, tasks, ake, ap, mseg, mlen, plw, S.deposit,
                                                             S.seg_q, track_all, mid);
             __syncwarp();
             s ^= 1;
@@ -204,8 +249,8 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
         }
 
         // ---- 2. the block's mesh and sums
-        const Acc128 k2 = acc_warp_sum(Acc128{(unsigned long long)ake, ake >> 63});
-        const Acc128 p2 = acc_warp_sum(Acc128{(unsigned long long)ap, ap >> 63});
+        const Acc128 k2 = i64_warp_sum(ake);
+        const Acc128 p2 = i64_warp_sum(ap);
         mseg = max(mseg, (unsigned)(((unsigned long long)mlen * (unsigned)(nx << SIC_POS_WIND_BITS)) >> 16));
         mseg = __reduce_max_sync(0xffffffffu, mseg);
         if (lane == 0) {
@@ -220,8 +265,8 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
             if (bad)
                 atomicOr(&sh.step_err, bad);
         }
-        // the new positions and velocities are read by the next step's bulk copies
-        asm volatile("fence.proxy.async;" ::: "memory");
+        if (!kept)  // the new positions and velocities are read by the next step's bulk copies
+            asm volatile("fence.proxy.async;" ::: "memory");
         __syncthreads();
         const bool diffs = sh.diff_used != 0;
         if (diffs)
@@ -309,13 +354,18 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
         if (S.refine_seg > 0 && mm > S.refine_seg)
             hold |= SIC_HOLD_REFINE;
         const bool last = hold || st + 1 == A.n_steps;
-        src ^= 1;
-        if (!last && first < n_items && lane == 0) {
-            asm volatile("fence.proxy.async;" ::: "memory");
-            issue(first, s, src);
-            if (claims && own == 1)
-                claimed = atomicAdd(&ctl->cursor[nxt_buf], 1u);
-        }
+        if (!kept)
+            src ^= 1;
+        // the next step's first item comes in during the field solve
+        auto next_item = [&]() {
+            if (!kept && !last && busy && lane == 0) {
+                asm volatile("fence.proxy.async;" ::: "memory");
+                stage_issue<PER_Q>(sh.own[warp], S.U[src], S.V[src], Qh, my_stage + s * WarpBuf<PER_Q, true>::stage,
+                                   &sh.mbar[warp][s]);
+                if (claims && own == 1)
+                    claimed = atomicAdd(&ctl->cursor[nxt_buf], 1u);
+            }
+        };
         if (last && !recorder)
             break;
 
@@ -332,6 +382,8 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 mv[k] = j + k < j1 ? (G > 1 ? __ldcg(mesh + j + k) : hist.get(j + k)) : 0ull;
+            if (j == j0)
+                next_item();
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (j + k < j1) {
@@ -341,6 +393,8 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
                     m1 += (__int128)(j + k) * (long long)mv[k];
                 }
         }
+        if (j0 == j1)  // (a thread without a cell)
+            next_item();
         long long incl = lsum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -368,16 +422,17 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
             M1 += make_i128(sh.hi[w], sh.lo[w]);
         }
         const __int128 sumD = (__int128)((long long)nx * (nx - 1) / 2) * qtot - (__int128)nx * M1;
-        __int128 D = (__int128)nx * (incl - lsum + before) - (__int128)j0 * qtot;
-        __int128 K = (__int128)nx * D - sumD;
+        // K_j = nx D_j - sumD, from cell to cell K_{j+1} = K_j + nx^2 mesh_j - nx Q
+        __int128 K = (__int128)nx * ((__int128)nx * (incl - lsum + before) - (__int128)j0 * qtot) - sumD;
+        const long long nx2 = (long long)nx * nx;
+        const __int128 nxq = (__int128)nx * qtot;
         const bool nodes = GEN && S.deposit == SIC_DEPOSIT_FIRST;
         const int mode_k = recorder ? S.mode_k : 0;
         float wloc = 0.f, mre = 0.f, mim = 0.f;
 #pragma unroll 1
         for (int j = j0; j < j1; ++j) {
             const long long m = (long long)hist.get(j);
-            D += (__int128)nx * m - qtot;
-            const __int128 Kn = (__int128)nx * D - sumD;
+            const __int128 Kn = K + (__int128)nx2 * m - nxq;
             const Norm128 nk = norm128(nodes ? K + Kn : K);
             ek[j].x = __fmul_rn(norm_to_float(nk, S.ek_exp - (nodes ? 1 : 0)), S.ek_mant);
             if (recorder) {
@@ -487,6 +542,27 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
         }
         if (last)
             break;
+    }
+    if (kept && busy && !timed_out) {
+        // the item back where it came from
+        const WorkItem W = sh.own[warp];
+        const int l0 = lane * R, mine = min(R, W.count - l0);
+        const unsigned *bu = reinterpret_cast<const unsigned *>(my_stage) + l0;
+        const float *bv = reinterpret_cast<const float *>(my_stage + kStageBytesU) + l0;
+        unsigned *U = S.U[src] + W.t0 + l0;
+        float *V = S.V[src] + W.t0 + l0;
+        if (mine == R) {
+#pragma unroll
+            for (int k = 0; k < R / 4; ++k) {
+                reinterpret_cast<uint4 *>(U)[k] = reinterpret_cast<const uint4 *>(bu)[k];
+                reinterpret_cast<float4 *>(V)[k] = reinterpret_cast<const float4 *>(bv)[k];
+            }
+        } else {
+            for (int r = 0; r < mine; ++r) {
+                U[r] = bu[r];
+                V[r] = bv[r];
+            }
+        }
     }
     if (G == 1)
         return;

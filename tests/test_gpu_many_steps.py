@@ -32,6 +32,7 @@ PROBLEMS = {
     "ragged": lambda: _tiny(6, 40, 3000, 300),
     "fewer tracers than cells": lambda: _tiny(7, 6, 300, 4096),
     "more items than warps": lambda: inputs.landau(0.3, 0.5, 512, 330, 2300, t_end=1.0),
+    "several rounds of items": lambda: inputs.landau(0.3, 0.5, 200, 1200, 1999, t_end=1.0),
 }
 
 
