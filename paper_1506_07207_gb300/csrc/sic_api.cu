@@ -13,6 +13,7 @@
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -209,14 +210,127 @@ int scalars_status(const SimScalars &sc);
 }
 namespace {
 
+// Pinned host memory for what a call reads back, lent for the call: copies
+// into a caller's pageable memory are staged by the driver one at a time, each
+// with a synchronisation of its own; into pinned memory they queue on the
+// stream behind the kernels, and the call synchronises once (us per call, before
+// and after: history 27 and 16, field 40 and 29, deposit 91 and 62, spectrum 55
+// and 43).  At most kPinnedKept buffers are kept for
+// later calls, of any thread; more are freed when they come back.
+constexpr size_t kPinnedBytes = 256 * 1024;
+constexpr int kPinnedKept = 4;
+
+std::mutex g_pinned_mu;
+void *g_pinned[kPinnedKept];
+int g_pinned_n = 0;
+
+class Pinned {
+public:
+    Pinned()
+    {
+        {
+            std::lock_guard<std::mutex> lock(g_pinned_mu);
+            if (g_pinned_n > 0)
+                p_ = g_pinned[--g_pinned_n];
+        }
+        if (!p_) {
+            // (allowed while another thread captures a stream)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            if (cudaHostAlloc(&p_, kPinnedBytes, cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                p_ = nullptr;
+            }
+            cudaThreadExchangeStreamCaptureMode(&mode);
+        }
+    }
+    ~Pinned()
+    {
+        if (!p_)
+            return;
+        {
+            std::lock_guard<std::mutex> lock(g_pinned_mu);
+            if (g_pinned_n < kPinnedKept) {
+                g_pinned[g_pinned_n++] = p_;
+                return;
+            }
+        }
+        cudaFreeHost(p_);
+    }
+    Pinned(const Pinned &) = delete;
+    Pinned &operator=(const Pinned &) = delete;
+
+    // Queue a copy of n bytes from the device into the buffer; nullptr when
+    // they do not fit (any more)
+    const char *queue(const void *dev, size_t n, cudaStream_t s, cudaError_t &e)
+    {
+        const size_t at = (used_ + 15) / 16 * 16;
+        if (!p_ || n > kPinnedBytes || at > kPinnedBytes - n)
+            return nullptr;
+        char *to = static_cast<char *>(p_) + at;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(to, dev, n, cudaMemcpyDeviceToHost, s);
+        used_ = at + n;
+        return to;
+    }
+
+private:
+    void *p_ = nullptr;
+    size_t used_ = 0;
+};
+
+// The arrays a call reads back, with the simulation's scalars, in one
+// synchronisation: add() each array (device address, bytes, the caller's
+// memory), then fetch().  Arrays that do not fit the pinned buffer are copied
+// the plain way.
+class Readback {
+public:
+    explicit Readback(sic_sim *sim) : sim_(sim) {}
+    void add(const void *dev, size_t n, void *to)
+    {
+        if (!to || n == 0)
+            return;
+        const char *from = parts_ < kMostParts ? pin_.queue(dev, n, sim_->stream, e_) : nullptr;
+        if (from)
+            later_[parts_++] = {from, n, to};
+        else if (e_ == cudaSuccess)
+            e_ = cudaMemcpyAsync(to, dev, n, cudaMemcpyDeviceToHost, sim_->stream);
+    }
+    // the SIC_E* code of the copies and of the device error bits
+    int fetch(SimScalars *out = nullptr)
+    {
+        SimScalars sc{};
+        add(sim_->h.sc, sizeof(sc), &sc);
+        const cudaError_t e = cudaStreamSynchronize(sim_->stream);  // (always: queued copies end here)
+        if (e_ == cudaSuccess)
+            e_ = e;
+        if (e_ != cudaSuccess)
+            return fail_cuda(sim_, e_);
+        for (int i = 0; i < parts_; ++i)
+            std::memcpy(later_[i].to, later_[i].from, later_[i].n);
+        if (out)
+            *out = sc;
+        return sic_host::scalars_status(sc);
+    }
+
+private:
+    struct Part {
+        const char *from;
+        size_t n;
+        void *to;
+    };
+    sic_sim *sim_;
+    Pinned pin_;
+    static constexpr int kMostParts = 4;
+    Part later_[kMostParts];
+    int parts_ = 0;
+    cudaError_t e_ = cudaSuccess;
+};
+
 int check_device_errors(sic_sim *sim, SimScalars *out = nullptr)
 {
-    SimScalars sc;
-    CK(cudaMemcpyAsync(&sc, sim->h.sc, sizeof(sc), cudaMemcpyDeviceToHost, sim->stream));
-    CK(cudaStreamSynchronize(sim->stream));
-    if (out)
-        *out = sc;
-    return sic_host::scalars_status(sc);
+    Readback rb(sim);
+    return rb.fetch(out);
 }
 
 // Clear the refinement hold of a synchronised simulation (the epilogue sets it
@@ -429,10 +543,10 @@ void free_plan(Plan &p, cudaStream_t s)
 }
 
 // A simulation of this many items or fewer runs on one block, its mesh in
-// shared memory: two items a warp cost less than adding two blocks' meshes
-// through L2 and waiting (16 items, 64 cells: 6.2 us a step on one block, 6.8
-// on two).
-constexpr int kOneBlockItems = 16;
+// shared memory; more take an item a warp on several blocks, which add their
+// meshes through L2 and wait (16 items, 64 cells: 6.3 us a step with two items
+// a warp on one block, 5.6 on two blocks).
+constexpr int kOneBlockItems = 8;
 
 // The groups of blocks of a launch of many steps (k_run), one per simulation:
 // block_begin[slot], and the grid; 0 when the steps are better launched one
@@ -933,12 +1047,10 @@ int sic_deposit(sic_sim *sim, int64_t *mesh_fixed_host, double *rho_host)
         return SIC_EINVAL;
     CK(launch(sim->plan, MODE_DEPOSIT, 0.0f, 0, 0, sim->stream));
     CK(launch_field_out(sim->h, sim->stream));
-    if (mesh_fixed_host)
-        CK(cudaMemcpyAsync(mesh_fixed_host, sim->h.mesh_last, 8 * (size_t)sim->nx, cudaMemcpyDeviceToHost,
-                           sim->stream));
-    if (rho_host)
-        CK(cudaMemcpyAsync(rho_host, sim->h.rho64, 8 * (size_t)sim->nx, cudaMemcpyDeviceToHost, sim->stream));
-    return check_device_errors(sim);
+    Readback rb(sim);
+    rb.add(sim->h.mesh_last, 8 * (size_t)sim->nx, mesh_fixed_host);
+    rb.add(sim->h.rho64, 8 * (size_t)sim->nx, rho_host);
+    return rb.fetch();
 }
 
 int sic_moments(sic_sim *sim, int32_t weighting, double *n_host, double *j_host)
@@ -949,11 +1061,10 @@ int sic_moments(sic_sim *sim, int32_t weighting, double *n_host, double *j_host)
     // rewrite them before reading them
     CK(launch_moments(sim->h, weighting, sim->L, 1.0 / sim->sigma, sim->L / (sim->dt * kPosUnits), sim->h.rho64,
                       sim->h.E64, sim->stream));
-    if (n_host)
-        CK(cudaMemcpyAsync(n_host, sim->h.rho64, 8 * (size_t)sim->nx, cudaMemcpyDeviceToHost, sim->stream));
-    if (j_host)
-        CK(cudaMemcpyAsync(j_host, sim->h.E64, 8 * (size_t)sim->nx, cudaMemcpyDeviceToHost, sim->stream));
-    return check_device_errors(sim);
+    Readback rb(sim);
+    rb.add(sim->h.rho64, 8 * (size_t)sim->nx, n_host);
+    rb.add(sim->h.E64, 8 * (size_t)sim->nx, j_host);
+    return rb.fetch();
 }
 
 int sic_refine(sic_sim *sim, double l_ref, int64_t *n_added)
@@ -1125,8 +1236,9 @@ int sic_field(sic_sim *sim, double *E_host)
     if (!sim || !E_host)
         return SIC_EINVAL;
     CK(launch_field_out(sim->h, sim->stream));
-    CK(cudaMemcpyAsync(E_host, sim->h.E64, 8 * (size_t)sim->nx, cudaMemcpyDeviceToHost, sim->stream));
-    return check_device_errors(sim);
+    Readback rb(sim);
+    rb.add(sim->h.E64, 8 * (size_t)sim->nx, E_host);
+    return rb.fetch();
 }
 
 int sic_push(sic_sim *sim)
@@ -1485,7 +1597,14 @@ int sic_diagnostics(sic_sim *sim, sic_diag *out)
     if (!sim || !out)
         return SIC_EINVAL;
     SimScalars sc;
-    int rc = check_device_errors(sim, &sc);
+    // the latest row with the scalars, while the ring is short enough to copy
+    // whole (which row it is they say)
+    constexpr int kShortRing = 256;
+    double ring[4 * kShortRing];
+    Readback rb(sim);
+    if (sim->hist_len <= kShortRing)
+        rb.add(sim->h.hist, 32 * (size_t)sim->hist_len, ring);
+    int rc = rb.fetch(&sc);
     if (rc)
         return rc;
     out->step = sc.step;
@@ -1496,7 +1615,15 @@ int sic_diagnostics(sic_sim *sim, sic_diag *out)
     if (sc.step > 0) {
         double row[4];
         const int64_t r = (sc.step - 1) % sim->hist_len;
-        CK(cudaMemcpy(row, sim->h.hist + 4 * r, sizeof(row), cudaMemcpyDeviceToHost));
+        if (sim->hist_len <= kShortRing) {
+            std::memcpy(row, ring + 4 * r, sizeof(row));
+        } else {
+            Readback rb2(sim);
+            rb2.add(sim->h.hist + 4 * r, sizeof(row), row);
+            rc = rb2.fetch();
+            if (rc)
+                return rc;
+        }
         out->kinetic_energy = row[1];
         out->momentum = row[2];
     }
@@ -1511,12 +1638,13 @@ int sic_history(sic_sim *sim, double *hist_host, int32_t max_rows, int32_t *rows
     if (!sim || !hist_host || !rows || max_rows < 1)
         return SIC_EINVAL;
     SimScalars sc;
-    int rc = check_device_errors(sim, &sc);
+    std::vector<double> ring(4 * (size_t)sim->hist_len);
+    Readback rb(sim);
+    rb.add(sim->h.hist, 8 * ring.size(), ring.data());
+    int rc = rb.fetch(&sc);
     if (rc)
         return rc;
     const int64_t n = std::min<int64_t>(std::min<int64_t>(sc.step, sim->hist_len), max_rows);
-    std::vector<double> ring(4 * (size_t)sim->hist_len);
-    CK(cudaMemcpy(ring.data(), sim->h.hist, 8 * ring.size(), cudaMemcpyDeviceToHost));
     for (int64_t i = 0; i < n; ++i) {
         const int64_t step = sc.step - n + i;
         std::memcpy(hist_host + 4 * i, ring.data() + 4 * (step % sim->hist_len), 32);
@@ -1530,12 +1658,13 @@ int sic_mode_history(sic_sim *sim, double *out_host, int32_t max_rows, int32_t *
     if (!sim || !out_host || !rows || max_rows < 1 || sim->mode_k <= 0)
         return SIC_EINVAL;
     SimScalars sc;
-    int rc = check_device_errors(sim, &sc);
+    std::vector<double> ring((size_t)sim->hist_len);
+    Readback rb(sim);
+    rb.add(sim->h.mhist, 8 * ring.size(), ring.data());
+    int rc = rb.fetch(&sc);
     if (rc)
         return rc;
     const int64_t n = std::min<int64_t>(std::min<int64_t>(sc.step, sim->hist_len), max_rows);
-    std::vector<double> ring((size_t)sim->hist_len);
-    CK(cudaMemcpy(ring.data(), sim->h.mhist, 8 * ring.size(), cudaMemcpyDeviceToHost));
     for (int64_t i = 0; i < n; ++i)
         out_host[i] = ring[(size_t)((sc.step - n + i) % sim->hist_len)];
     *rows = (int32_t)n;
@@ -1548,8 +1677,9 @@ int sic_spectrum(sic_sim *sim, int32_t field, double *out_host)
         return SIC_EINVAL;
     CK(launch_field_out(sim->h, sim->stream));
     CK(launch_spectrum(sim->h, field, sim->stream));
-    CK(cudaMemcpyAsync(out_host, sim->h.spec, 8 * (size_t)(sim->nx / 2 + 1), cudaMemcpyDeviceToHost, sim->stream));
-    return check_device_errors(sim);
+    Readback rb(sim);
+    rb.add(sim->h.spec, 8 * (size_t)(sim->nx / 2 + 1), out_host);
+    return rb.fetch();
 }
 
 int sic_get_state(sic_sim *sim, double *x_host, double *v_host)
@@ -1563,8 +1693,12 @@ int sic_get_state(sic_sim *sim, double *x_host, double *v_host)
     const int b = sc.buf & 1;
     std::vector<uint32_t> U(sim->n_alloc);
     std::vector<float> V(sim->n_alloc);
-    CK(cudaMemcpy(U.data(), sim->h.U[b], 4 * U.size(), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(V.data(), sim->h.V[b], 4 * V.size(), cudaMemcpyDeviceToHost));
+    Readback rb(sim);
+    rb.add(sim->h.U[b], 4 * U.size(), U.data());
+    rb.add(sim->h.V[b], 4 * V.size(), V.data());
+    rc = rb.fetch();
+    if (rc)
+        return rc;
     // each sheet unwrapped along its tracers: the first one inside the box,
     // every next one a segment (the 32-bit position difference) further
     const double unit = sim->L / kPosUnits, vs = sim->L / (sim->dt * kPosUnits);
@@ -1664,8 +1798,6 @@ int64_t sic_launch_count(void) { return sic::launches(); }
 // file-scope device array instead of a per-call allocation.  The paper has no
 // counterpart; this serves callers that must not allocate device memory while
 // stepping.
-
-#include <mutex>
 
 namespace {
 
