@@ -703,7 +703,7 @@ struct Shared {
     // k_run: the step's longest segment and error bits, the block's sums, and
     // whether the wait for the other blocks gave up
     unsigned long long step_mseg;
-    unsigned step_err, gave_up;
+    unsigned step_err, gave_up, last_out;
     unsigned long long tot[2][2];  // KE, P: lo, hi
     WorkItem own[NW];              // each warp's first item of a step
     Beside beside[NW];

@@ -1,6 +1,8 @@
 // sic_run.cu -- k_run: many steps of one or many simulations in one
 // cooperative launch (sic_step, sic_run, batches and the server take it where
 // a step is short; k_step of sic_kernels.cu has one launch a step).
+#include <mutex>
+
 #include "sic_item.cuh"
 
 namespace sic {
@@ -566,18 +568,24 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
     }
     if (G == 1)
         return;
-    // the last step is over and its buffers are read by no block but the
-    // recorder, which is done with them: leave the mesh, the sums and the
-    // block count clear for the next launch
-    if (recorder) {
-        for (int j = tid; j < nx; j += B)
-            S.mesh[j] = 0ull;
-        for (int i = tid; i < (int)(sizeof(ctl->acc) / 8); i += B)
-            reinterpret_cast<unsigned long long *>(ctl->acc)[i] = 0ull;
-        if (tid < 3)
-            ctl->cursor[tid] = 0u;
+    // Leave the mesh, the sums and the block count clear for the next launch.
+    // The last block out does it: until a block is counted here it may still
+    // be reading the last step's sums, and the recorder its mesh.
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        sh.last_out = atomicAdd(&ctl->out, 1u) + 1 == (unsigned)G;
     }
-    if (tid == 0 && atomicAdd(&ctl->out, 1u) + 1 == (unsigned)G) {
+    __syncthreads();
+    if (!sh.last_out)
+        return;
+    for (int j = tid; j < nx; j += B)
+        S.mesh[j] = 0ull;
+    for (int i = tid; i < (int)(sizeof(ctl->acc) / 8); i += B)
+        reinterpret_cast<unsigned long long *>(ctl->acc)[i] = 0ull;
+    if (tid < 3)
+        ctl->cursor[tid] = 0u;
+    if (tid == 3) {
         ctl->out = 0u;
         ctl->bar = 0u;
     }
@@ -613,7 +621,9 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_run(const RunArgs A)
 template <int Q, bool G>
 cudaError_t prep_run(size_t smem)
 {
+    static std::mutex mu;  // (two threads' first calls: the attribute only grows)
     static size_t done = 0;
+    std::lock_guard<std::mutex> lock(mu);
     if (smem > done) {
         const cudaError_t e =
             cudaFuncSetAttribute(k_run<Q, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
