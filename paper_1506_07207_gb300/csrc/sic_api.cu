@@ -1059,8 +1059,8 @@ int sic_moments(sic_sim *sim, int32_t weighting, double *n_host, double *j_host)
         return SIC_EINVAL;
     // E64 and rho64 serve as the device buffers: sic_field and sic_deposit
     // rewrite them before reading them
-    CK(launch_moments(sim->h, weighting, sim->L, 1.0 / sim->sigma, sim->L / (sim->dt * kPosUnits), sim->h.rho64,
-                      sim->h.E64, sim->stream));
+    CK(launch_moments(sim->h, sim->n_alloc, weighting, sim->L, 1.0 / sim->sigma, sim->L / (sim->dt * kPosUnits),
+                      sim->h.rho64, sim->h.E64, sim->stream));
     Readback rb(sim);
     rb.add(sim->h.rho64, 8 * (size_t)sim->nx, n_host);
     rb.add(sim->h.E64, 8 * (size_t)sim->nx, j_host);
