@@ -290,8 +290,9 @@ int sic_step(sic_sim *sim, int32_t n_steps);
 int sic_step_batch(sic_sim *const *sims, int32_t n_sims, const int32_t *n_steps);
 
 /* A persistent batch: its launch plan is built once, so stepping it costs
- * one kernel launch per step for all members (CUDA graphs of 8 steps when
- * n_steps >= 8).  While the batch exists its members must be advanced only
+ * at most one kernel launch per step and charge mode for all members (CUDA
+ * graphs of 8 steps when n_steps >= 8), or one for up to 256 steps where the
+ * members are small enough.  While the batch exists its members must be advanced only
  * through it; it runs on the first member's stream, ordered after all
  * members' streams at create and before them at destroy.  Every member
  * advances by the same number of steps; results equal sic_step bit for bit. */
@@ -383,8 +384,9 @@ int64_t sic_launch_count(void);
  * sic_create_horizontal) and a step count.  Requests wait in arrival order;
  * the server admits waiting requests while an active slot is free and their
  * device memory fits the budget, advances all active simulations together by
- * up to chunk_steps steps (each step is one kernel launch over all of them,
- * a second one for simulations that carry per-particle charges), and retires
+ * up to chunk_steps steps (one kernel launch for all of them where the
+ * simulations are small enough; else each step is one launch, and a second one
+ * for simulations that carry per-particle charges), and retires
  * the finished ones.  A request that holds for refinement (Sec. 2.6) is
  * refined and goes on.  The batched mode overlaps its host work with the
  * GPU: a tick waits for the chunk launched by the tick before, launches the
