@@ -941,10 +941,13 @@ namespace {
 // into FP64 by their bits, and the reciprocal of the length is one
 // third-order step from the FP32 one.  The diagnostics of 512 x 2048 folded
 // tracers on 512 cells (both orders, a deposit, the field and two spectra) take
-// 0.48 ms, of which the moments 99 and 211 us as calls; 0.72 ms with one mesh
+// 0.47 ms, of which the moments 98 and 199 us as calls; 0.72 ms with one mesh
 // for all blocks, 1.59 ms with every cell's share worked out as well, 49.5 ms
 // with one thread per work item.
 constexpr int kMomentCells = 8;
+// Two warps a block: items differ in cost by their cells, and small blocks leave
+// a shorter tail (first order 211 us a call with eight warps)
+constexpr int kMomentThreads = 64;
 
 // v 2^-32 for v < 2^52, exactly: one FP64 subtraction instead of a conversion
 __device__ __forceinline__ double cells_double(unsigned long long v)
@@ -1013,7 +1016,7 @@ struct MomentRun {
 };
 
 template <int W>
-__global__ void __launch_bounds__(256) k_moments(const SimDev S, double inv_dx, double unit_q, double unit_v, double *n,
+__global__ void __launch_bounds__(kMomentThreads) k_moments(const SimDev S, double inv_dx, double unit_q, double unit_v, double *n,
                                                  double *j, int copies)
 {
     const int nx = S.nx, nx4 = nx << SIC_POS_WIND_BITS;
@@ -1293,13 +1296,15 @@ cudaError_t launch_moments(const SimDev &sim, long long n_alloc, int weighting, 
     }
     if (e != cudaSuccess)
         return e;
-    // one warp per work item, blocks of 8 warps
-    const int grid = (int)std::max<long long>(1, std::min<long long>(16384, ((long long)sim.n_items + 7) / 8));
+    // one warp per work item
+    constexpr int warps = kMomentThreads / 32;
+    const int grid =
+        (int)std::max<long long>(1, std::min<long long>(131072 / warps, ((long long)sim.n_items + warps - 1) / warps));
     const double inv_dx = (double)sim.nx / box_length;
     if (weighting == 0)
-        k_moments<0><<<grid, 256, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, copies);
+        k_moments<0><<<grid, kMomentThreads, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, copies);
     else
-        k_moments<1><<<grid, 256, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, copies);
+        k_moments<1><<<grid, kMomentThreads, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, copies);
     if (copies > 1)
         k_moments_sum<<<(sim.nx + 255) / 256, 256, 0, s>>>(sim, n, j, copies);
     count_launches(1);
