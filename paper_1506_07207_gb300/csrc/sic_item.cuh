@@ -493,22 +493,45 @@ struct Spill {
     unsigned err;
 };
 
-// The rare path of sum_add: the lane's sum goes into the block's 128-bit sum
-// (shared memory), and so does the term y unless it fits a fresh 64-bit sum.
-// y is integer-valued when it is 2^63 or more (below 2^124; inf, NaN or
-// larger set bit 31 of the error word instead).
-__device__ __noinline__ Spill acc_spill(long long a, float y, unsigned long long *blk)
+// The rare path of sum_add, for the whole warp: the sums of the lanes that ask
+// for it go into the block's 128-bit sum (shared memory), and so do their terms
+// y unless they fit a fresh 64-bit sum.  y is integer-valued when it is 2^63 or
+// more (below 2^124; inf, NaN or larger set bit 31 of the error word instead).
+// The lanes are summed first: plasmas that start at rest have units so fine
+// that every lane comes here, and 256 64-bit adds to one word, loops of
+// compare-and-swap, were most of their step (a cold oscillation of 4096 tracers
+// on 64 cells, us a step: 26.3 lane by lane, 6.3).
+__device__ __noinline__ Spill acc_spill(long long a, float y, unsigned long long *blk, bool mine)
 {
-    atomic_add_i128(blk, (__int128)a);
-    if (fabsf(y) < 9223372036854775808.0f)
-        return Spill{__float2ll_rz(y), 0u};
-    const unsigned b = __float_as_uint(y);
-    const int sh = (int)((b >> 23) & 0xffu) - 150;  // y = m 2^sh, sh >= 40 here
-    if (sh > 100)
-        return Spill{0, 0x80000000u};
-    const __int128 m = (__int128)((b & 0x7fffffu) | 0x800000u) << sh;
-    atomic_add_i128(blk, (b >> 31) ? -m : m);
-    return Spill{0, 0u};
+    Spill r{a, 0u};
+    Acc128 t{0ull, 0ll};
+    if (mine) {
+        r.a = 0;
+        __int128 v = a;
+        if (fabsf(y) < 9223372036854775808.0f) {
+            r.a = __float2ll_rz(y);
+        } else {
+            const unsigned b = __float_as_uint(y);
+            const int sh = (int)((b >> 23) & 0xffu) - 150;  // y = m 2^sh, sh >= 40 here
+            if (sh > 100) {
+                r.err = 0x80000000u;
+            } else {
+                const __int128 m = (__int128)((b & 0x7fffffu) | 0x800000u) << sh;
+                v += (b >> 31) ? -m : m;
+            }
+        }
+        t = Acc128{(unsigned long long)v, (long long)(v >> 64)};
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Acc128 b;
+        b.lo = __shfl_down_sync(0xffffffffu, t.lo, o);
+        b.hi = __shfl_down_sync(0xffffffffu, t.hi, o);
+        acc_add(t, b);
+    }
+    if ((threadIdx.x & 31) == 0)
+        atomic_add_i128(blk, (__int128)(((unsigned __int128)(unsigned long long)t.hi << 64) | t.lo));
+    return r;
 }
 
 // Add y (a term already in the sum's fixed-point unit), truncated to an
@@ -525,9 +548,10 @@ __device__ __forceinline__ void sum_add(long long &a, float y, unsigned long lon
     const int l = __float2int_rz(__fmaf_rn(__int2float_rn(h), -0x1p22f, y));
     const long long v = (long long)h * (1ll << 22) + l;
     const long long s = (long long)((unsigned long long)a + (unsigned long long)v);
-    if (__builtin_expect(!(fabsf(y) < 9007199254740992.0f) || ((a ^ s) & (v ^ s)) < 0, 0)) {
-        const Spill r = acc_spill(a, y, blk);
-        a = r.a;
+    const bool over = !(fabsf(y) < 9007199254740992.0f) || ((a ^ s) & (v ^ s)) < 0;
+    if (__builtin_expect(__any_sync(0xffffffffu, over), 0)) {
+        const Spill r = acc_spill(a, y, blk, over);
+        a = over ? r.a : s;
         err |= r.err;
     } else {
         a = s;
