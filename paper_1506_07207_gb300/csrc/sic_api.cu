@@ -607,6 +607,18 @@ static int split_blocks(sic_sim *const *sims, int n, int nx_max, int charges, bo
     return block_begin[n];
 }
 
+// The second and third mesh of every simulation of a k_run launch, in the plan's
+// memory at `at` (16 nx_max bytes each; k_run clears a mesh before it is used)
+static void set_run_meshes(std::vector<SimDev> &table, char *at, int nx_max)
+{
+    unsigned long long *mesh = (unsigned long long *)at;
+    for (SimDev &d : table)
+        for (unsigned long long *&m : d.run_mesh) {
+            m = mesh;
+            mesh += nx_max;
+        }
+}
+
 // Build the device plan of one launch over several simulations (slot order):
 // the table of their descriptors, where each one's items start in the
 // launch's list, and the zeroed claim cursors, item tickets and block count.
@@ -657,10 +669,13 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     const size_t oK = lay.take(4 * (size_t)(2 * n + 1));  // cursor[n], tickets[n], done
     const size_t oC = p.run_grid ? lay.take(sizeof(RunCtl) * (size_t)n) : lay.off;
     const size_t cleared = lay.off - oK;
+    const size_t oM = p.run_grid ? lay.take(16 * (size_t)n * nx_max) : 0;
     cudaError_t e = cudaMallocAsync(&p.mem, lay.off, s);
     if (e != cudaSuccess)
         return e;
     char *b = (char *)p.mem;
+    if (p.run_grid)
+        set_run_meshes(table, b + oM, nx_max);
     e = cudaMemcpyAsync(b + oT, table.data(), sizeof(SimDev) * table.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b + oS, slot_begin.data(), 4 * slot_begin.size(), cudaMemcpyHostToDevice, s);
@@ -710,6 +725,7 @@ cudaError_t build_many_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s
     const size_t oT = lay.take(sizeof(SimDev) * table.size());
     const size_t oB = lay.take(4 * block_begin.size());
     const size_t oC = lay.take(sizeof(RunCtl) * (size_t)n);
+    const size_t oM = lay.take(16 * (size_t)n * nx_max);
     cudaError_t e = cudaMallocAsync(&p.mem, lay.off, s);
     if (e != cudaSuccess) {
         p.mem = nullptr;
@@ -717,6 +733,7 @@ cudaError_t build_many_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s
         return e;
     }
     char *b = (char *)p.mem;
+    set_run_meshes(table, b + oM, nx_max);
     e = cudaMemcpyAsync(b + oT, table.data(), sizeof(SimDev) * table.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b + oB, block_begin.data(), 4 * block_begin.size(), cudaMemcpyHostToDevice, s);

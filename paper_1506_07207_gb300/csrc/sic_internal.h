@@ -24,6 +24,9 @@
 //                        shared memory).
 //   E64[nx]       double the node field E_j in physical units.
 //   rho64[nx]     double the neutralised density of the latest deposit.
+//                        (Both are written for the host on request only, and no
+//                        step touches them: a member of a batch may be read on
+//                        its own stream while the batch steps it.)
 // Charge unit: a segment between tracers of weights w_i, w_{i+1} carries
 // Q_s = Qh_i + Qh_{i+1} = round(w_i sigma / 2) + round(w_{i+1} sigma / 2)
 // units, sigma a power of two chosen so that every Q_s <= 2^28.
@@ -155,6 +158,8 @@ struct SimDev {
     double *spec;               // [nx / 2 + 1] Fourier amplitudes (sic_spectrum)
     int32_t mode_k;             // 0: no mode history
     int32_t pad2;
+    unsigned long long *run_mesh[2];  // k_run's second and third mesh: the launch plan's own,
+                                      // set in its table alone
 };
 
 // Everything one launch of the step kernel needs.

@@ -40,8 +40,8 @@ __device__ __forceinline__ bool group_wait(const unsigned *bar, unsigned target)
 //      its way; the group's last block also records the step.
 // A group of one block keeps the mesh in shared memory.  The mesh and the
 // sums have three buffers: the one of step i is cleared during step i + 2,
-// when every block has read it.  E64 and rho64, which only hold what
-// k_field_out writes on request, serve as the second and third mesh.
+// when every block has read it.  The second and third mesh are the plan's own:
+// nothing that a call reading the simulation on another stream writes is theirs.
 //
 // us per step in runs of 160 steps, graphs of single steps and this: 4 K
 // tracers 9.8 and 6.3, 262 K 10.8 and 5.7, 430 K irregular 28 and 16, 8.4 M 41
@@ -221,7 +221,7 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
     for (int st = 0;; ++st) {
         const int now = st % 3, nxt_buf = (st + 1) % 3;
         auto mesh_of = [&](int k) {
-            return k == 0 ? S.mesh : reinterpret_cast<unsigned long long *>(k == 1 ? S.E64 : S.rho64);
+            return k == 0 ? S.mesh : S.run_mesh[k - 1];
         };
         if (G > 1 && recorder) {
             unsigned long long *m = mesh_of(nxt_buf);
