@@ -219,9 +219,8 @@ int sic_field(sic_sim *sim, double *E_host);
  *     velocity interpolated linearly between the tracers' velocities.
  * The velocities are the stored ones (v^{n-1/2} after a step), the charges
  * the fixed-point ones of the deposit.  Diagnostic only: FP64 with atomics,
- * equal to the FP64 definition within rounding but not bit-reproducible; a
- * particle longer than 64 box lengths is left out (the paper stops a run at
- * one box length, Sec. 3.2).  Other weightings: SIC_EINVAL.
+ * equal to the FP64 definition within rounding but not bit-reproducible.  Other
+ * weightings: SIC_EINVAL.
  */
 int sic_moments(sic_sim *sim, int32_t weighting, double *n_host, double *j_host);
 
@@ -293,9 +292,13 @@ int sic_step_batch(sic_sim *const *sims, int32_t n_sims, const int32_t *n_steps)
  * at most one kernel launch per step and charge mode for all members (CUDA
  * graphs of 8 steps when n_steps >= 8), or one for up to 256 steps where the
  * members are small enough.  While the batch exists its members must be advanced only
- * through it; it runs on the first member's stream, ordered after all
- * members' streams at create and before them at destroy.  Every member
- * advances by the same number of steps; results equal sic_step bit for bit. */
+ * through it (sic_push, sic_deposit and sic_refine change a member too); it runs
+ * on the first member's stream, ordered after all members' streams at create and
+ * before them at destroy.  Every member advances by the same number of steps;
+ * results equal sic_step bit for bit.  The calls that read a member (sic_field,
+ * sic_moments, sic_spectrum, sic_diagnostics, ...) never change its run; on a
+ * member with a stream of its own they are not ordered after the batch's steps,
+ * so sic_sync of the first member goes before a read of a certain step. */
 typedef struct sic_batch sic_batch;
 int sic_batch_create(sic_sim *const *sims, int32_t n_sims, sic_batch **out);
 int sic_batch_step(sic_batch *batch, int32_t n_steps);

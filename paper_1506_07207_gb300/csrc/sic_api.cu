@@ -1074,10 +1074,27 @@ int sic_moments(sic_sim *sim, int32_t weighting, double *n_host, double *j_host)
 {
     if (!sim || (weighting != 0 && weighting != 1))
         return SIC_EINVAL;
-    // E64 and rho64 serve as the device buffers: sic_field and sic_deposit
-    // rewrite them before reading them
-    CK(launch_moments(sim->h, sim->n_alloc, weighting, sim->L, 1.0 / sim->sigma, sim->L / (sim->dt * kPosUnits),
-                      sim->h.rho64, sim->h.E64, sim->stream));
+    // The copies are the simulation's own, nothing a step uses (a member of a
+    // batch may be read while it steps), and kept: at most 256 KB, which not
+    // every simulation needs.  Without room for them there are none.
+    int copies = moment_copies(sim->nx, (int64_t)sim->items.size());
+    const size_t bytes = 16 * (size_t)copies * (size_t)sim->nx;
+    if (copies > 1 && sim->moments_bytes < bytes) {  // (a refinement has added items, or the first call)
+        if (sim->moments)
+            cudaFreeAsync(sim->moments, sim->stream);
+        sim->moments_bytes = 0;
+        if (cudaMallocAsync(&sim->moments, bytes, sim->stream) == cudaSuccess) {
+            sim->moments_bytes = bytes;
+        } else {
+            cudaGetLastError();
+            sim->moments = nullptr;
+            copies = 1;
+        }
+    }
+    // E64 and rho64 serve as the results' device buffers: sic_field and
+    // sic_deposit rewrite them before reading them
+    CK(launch_moments(sim->h, (double *)sim->moments, copies, weighting, sim->L, 1.0 / sim->sigma,
+                      sim->L / (sim->dt * kPosUnits), sim->h.rho64, sim->h.E64, sim->stream));
     Readback rb(sim);
     rb.add(sim->h.rho64, 8 * (size_t)sim->nx, n_host);
     rb.add(sim->h.E64, 8 * (size_t)sim->nx, j_host);
@@ -1773,6 +1790,8 @@ void sic_destroy(sic_sim *sim)
         free_plan(sim->plan, sim->stream);
         if (sim->dmem)
             cudaFreeAsync(sim->dmem, sim->stream);
+        if (sim->moments)
+            cudaFreeAsync(sim->moments, sim->stream);
         cudaStreamSynchronize(sim->stream);
     }
     if (sim->own_stream && sim->stream)

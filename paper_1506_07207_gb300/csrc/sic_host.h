@@ -64,6 +64,8 @@ struct sic_sim {
     bool own_stream = false;
     void *dmem = nullptr;
     size_t dbytes = 0;
+    void *moments = nullptr;          // sic_moments' copies of n and j, from the first call that takes some
+    size_t moments_bytes = 0;
     SimDev h{};
     sic_host::Plan plan;
     cudaGraphExec_t gexec = nullptr;

@@ -221,8 +221,11 @@ cudaError_t launch_spectrum(const SimDev &sim, int field, cudaStream_t s);
 cudaError_t launch_refine_count(const SimDev &sim, long long lfix, int32_t *splits, cudaStream_t s);
 cudaError_t launch_refine_scatter(const SimDev &sim, long long lfix, const int64_t *out_base, uint32_t *U2, float *V2,
                                   int32_t *Q2, cudaStream_t s);
-cudaError_t launch_moments(const SimDev &sim, long long n_alloc, int weighting, double box_length, double unit_q, double unit_v,
-                           double *n, double *j, cudaStream_t s);
+// The copies of n and j that the moments' atomics are better spread over (1: none,
+// no scratch); scratch: 2 copies nx doubles
+int moment_copies(int nx, long long n_items);
+cudaError_t launch_moments(const SimDev &sim, double *scratch, int copies, int weighting, double box_length,
+                           double unit_q, double unit_v, double *n, double *j, cudaStream_t s);
 cudaError_t launch_expand_horizontal(uint32_t *U, float *V, const uint32_t *u_template, int32_t n_template,
                                      const float *v_sheet, const int64_t *sheet_offset, int32_t n_sheets,
                                      cudaStream_t s);

@@ -1015,9 +1015,12 @@ struct MomentRun {
     }
 };
 
+// scratch: `copies` times a copy of n and one of j beside it (262 K tracers on 128
+// cells: 74 and 79 us a call for the two orders with the copies in two arrays,
+// 61 and 73 so); one copy: n and j themselves
 template <int W>
 __global__ void __launch_bounds__(kMomentThreads) k_moments(const SimDev S, double inv_dx, double unit_q, double unit_v, double *n,
-                                                 double *j, int copies)
+                                                 double *j, double *scratch, int copies)
 {
     const int nx = S.nx, nx4 = nx << SIC_POS_WIND_BITS;
     const int lane = threadIdx.x & 31;
@@ -1026,8 +1029,8 @@ __global__ void __launch_bounds__(kMomentThreads) k_moments(const SimDev S, doub
     const float *V = S.V[src];
     const int32_t *Qh = S.Qh;
     if (copies > 1) {
-        n = reinterpret_cast<double *>(S.U[src ^ 1]) + (size_t)(blockIdx.x % copies) * nx;
-        j = reinterpret_cast<double *>(S.V[src ^ 1]) + (size_t)(blockIdx.x % copies) * nx;
+        n = scratch + (size_t)(blockIdx.x % copies) * 2 * nx;
+        j = n + nx;
     }
     const double q_unit = unit_q * inv_dx;  // charge units to density in one cell
     const int warps = (int)((gridDim.x * blockDim.x) >> 5);
@@ -1236,35 +1239,18 @@ __global__ void __launch_bounds__(kMomentThreads) k_moments(const SimDev S, doub
     }
 }
 
-// The copies of n and j in the buffers that the next step will write, cleared
-__global__ void __launch_bounds__(256) k_moments_clear(const SimDev S, int words)
+// The sums of the copies of n and j, in order
+__global__ void __launch_bounds__(256) k_moments_sum(int nx, const double *scratch, double *n, double *j, int copies)
 {
-    const int src = (int)S.sc->buf;
-    const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (i < words) {
-        reinterpret_cast<double *>(S.U[src ^ 1])[i] = 0.0;
-        reinterpret_cast<double *>(S.V[src ^ 1])[i] = 0.0;
-    }
-}
-
-// Their sums, in order; the copies are left clear (between sheets these
-// buffers hold zeros)
-__global__ void __launch_bounds__(256) k_moments_sum(const SimDev S, double *n, double *j, int copies)
-{
-    const int src = (int)S.sc->buf;
     const int c = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (c >= S.nx)
+    if (c >= nx)
         return;
-    double *cn = reinterpret_cast<double *>(S.U[src ^ 1]) + c, *cj = reinterpret_cast<double *>(S.V[src ^ 1]) + c;
+    const double *cn = scratch + c, *cj = cn + nx;
     double sn = 0.0, sj = 0.0;
 #pragma unroll 8
     for (int k = 0; k < copies; ++k) {
-        sn += cn[(size_t)k * S.nx];
-        sj += cj[(size_t)k * S.nx];
-    }
-    for (int k = 0; k < copies; ++k) {
-        cn[(size_t)k * S.nx] = 0.0;
-        cj[(size_t)k * S.nx] = 0.0;
+        sn += cn[(size_t)k * 2 * nx];
+        sj += cj[(size_t)k * 2 * nx];
     }
     n[c] = sn;
     j[c] = sj;
@@ -1274,21 +1260,21 @@ __global__ void __launch_bounds__(256) k_moments_sum(const SimDev S, double *n, 
 
 // On a small mesh all atomics meet in a few slices of the L2 (one 80 % busy,
 // the average 7 %: 229 and 298 us for the two orders on 512 cells), so blocks take turns with copies of n and j, kMomentWords
-// cells altogether, which lie where the next step writes its tracers: no block
-// shares a copy with all others, and nothing is allocated.  Not for few items
-// (a block for every copy) and where the copies do not fit.
+// cells altogether, in the caller's scratch: no block shares a copy with all
+// others.  Not for few items (a block for every copy) and without scratch.
 constexpr int kMomentWords = 16384;
 
-cudaError_t launch_moments(const SimDev &sim, long long n_alloc, int weighting, double box_length, double unit_q,
-                           double unit_v, double *n, double *j, cudaStream_t s)
+int moment_copies(int nx, long long n_items)
 {
-    long long most = std::min<long long>(kMomentWords / sim.nx, n_alloc / (2ll * sim.nx));
-    most = std::min(most, ((long long)sim.n_items + 7) / 8);
-    const int copies = (int)std::max(1ll, most);
+    return (int)std::max(1ll, std::min<long long>(kMomentWords / nx, (n_items + 7) / 8));
+}
+
+cudaError_t launch_moments(const SimDev &sim, double *scratch, int copies, int weighting, double box_length,
+                           double unit_q, double unit_v, double *n, double *j, cudaStream_t s)
+{
     cudaError_t e = cudaSuccess;
     if (copies > 1) {
-        k_moments_clear<<<(copies * sim.nx + 255) / 256, 256, 0, s>>>(sim, copies * sim.nx);
-        count_launches(2);
+        e = cudaMemsetAsync(scratch, 0, 2 * sizeof(double) * (size_t)copies * (size_t)sim.nx, s);
     } else {
         e = cudaMemsetAsync(n, 0, sizeof(double) * (size_t)sim.nx, s);
         if (e == cudaSuccess)
@@ -1302,12 +1288,14 @@ cudaError_t launch_moments(const SimDev &sim, long long n_alloc, int weighting, 
         (int)std::max<long long>(1, std::min<long long>(131072 / warps, ((long long)sim.n_items + warps - 1) / warps));
     const double inv_dx = (double)sim.nx / box_length;
     if (weighting == 0)
-        k_moments<0><<<grid, kMomentThreads, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, copies);
+        k_moments<0><<<grid, kMomentThreads, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, scratch, copies);
     else
-        k_moments<1><<<grid, kMomentThreads, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, copies);
-    if (copies > 1)
-        k_moments_sum<<<(sim.nx + 255) / 256, 256, 0, s>>>(sim, n, j, copies);
+        k_moments<1><<<grid, kMomentThreads, 0, s>>>(sim, inv_dx, unit_q, unit_v, n, j, scratch, copies);
     count_launches(1);
+    if (copies > 1) {
+        k_moments_sum<<<(sim.nx + 255) / 256, 256, 0, s>>>(sim.nx, scratch, n, j, copies);
+        count_launches(1);
+    }
     return cudaGetLastError();
 }
 

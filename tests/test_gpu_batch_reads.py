@@ -35,6 +35,8 @@ READS = {
     "field": lambda s: s.sic_field(),
     "density spectrum": lambda s: s.sic_spectrum(0),
     "field spectrum": lambda s: s.sic_spectrum(1),
+    "moments": lambda s: s.sic_moments(0),
+    "first-order moments": lambda s: s.sic_moments(1),
 }
 CALLS, STEPS = 12, 40
 
