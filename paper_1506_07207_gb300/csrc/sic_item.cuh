@@ -1292,6 +1292,10 @@ __device__ __forceinline__ void do_item(const WorkItem &W, const unsigned *__res
         // memory, so the cross-cell segments can be shared out over the warp
         unsigned *pts = reinterpret_cast<unsigned *>(st);
         int *qpts = reinterpret_cast<int *>(st + WarpBuf<PER_Q, STAGED>::q_offset);
+        // (every lane has written its tracers back there, the lane after the
+        // last one too, whose first words may be the halo's)
+        if (KEPT)
+            __syncwarp();
         if (FULL || rn == R) {
 #pragma unroll
             for (int k = 0; k < R / 4; ++k) {
