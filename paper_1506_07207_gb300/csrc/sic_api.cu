@@ -607,6 +607,11 @@ static int split_blocks(sic_sim *const *sims, int n, int nx_max, int charges, bo
     return block_begin[n];
 }
 
+// Polls of a block of k_run that waits for its group: about three seconds.
+// SIC_WAIT_POLLS, a test knob, makes the wait run out (the simulation ends with
+// SIC_ETIMEOUT).
+static int wait_polls() { return env_int("SIC_WAIT_POLLS", 1 << 22); }
+
 // The second and third mesh of every simulation of a k_run launch, in the plan's
 // memory at `at` (16 nx_max bytes each; k_run clears a mesh before it is used)
 static void set_run_meshes(std::vector<SimDev> &table, char *at, int nx_max)
@@ -700,7 +705,7 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
     p.args.gen = gen ? 1 : 0;
     p.grid = grid;
     p.per_q = per_q;
-    p.run = RunArgs{p.args.sims, (const int32_t *)(b + oB), (RunCtl *)(b + oC), n, nx_max, 0};
+    p.run = RunArgs{p.args.sims, (const int32_t *)(b + oB), (RunCtl *)(b + oC), n, nx_max, 0, wait_polls()};
     return cudaSuccess;
 }
 
@@ -741,7 +746,7 @@ cudaError_t build_many_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s
         e = cudaMemsetAsync(b + oC, 0, sizeof(RunCtl) * (size_t)n, s);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(s);  // host staging vectors go out of scope
-    p.run = RunArgs{(const SimDev *)(b + oT), (const int32_t *)(b + oB), (RunCtl *)(b + oC), n, nx_max, 0};
+    p.run = RunArgs{(const SimDev *)(b + oT), (const int32_t *)(b + oB), (RunCtl *)(b + oC), n, nx_max, 0, wait_polls()};
     return e;
 }
 

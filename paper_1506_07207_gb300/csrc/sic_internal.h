@@ -184,8 +184,9 @@ struct LaunchArgs {
                                  // 1: never; 2: whenever it fits (autotuning)
 };
 
-// What the blocks of one simulation share in a launch of k_run (all zero
-// between launches): the sums of three steps (SimAccum::pad[0]: error bits),
+// What the blocks of one simulation share in a launch of k_run (all zero between
+// launches, unless a block gave up waiting: that simulation holds with an error,
+// and a held one's blocks leave before they look here): the sums of three steps (SimAccum::pad[0]: error bits),
 // their claims of items, and the counts of blocks that have finished a step
 // and that have left.
 struct RunCtl {
@@ -205,6 +206,7 @@ struct RunArgs {
     int32_t n_slots;
     int32_t nx_max;
     int32_t n_steps;
+    int32_t wait_polls;          // a block gives up waiting for its group after this many polls
 };
 
 #include <cuda_runtime.h>

@@ -11,11 +11,11 @@ namespace {
 
 // ------------------------------------------------- many steps a launch ----
 
-// A bounded wait until *bar reaches target (modulo 2^32): false after about
-// three seconds (a poll is a trip to L2, about 0.7 us).
-__device__ __forceinline__ bool group_wait(const unsigned *bar, unsigned target)
+// A bounded wait until *bar reaches target (modulo 2^32): false after this many
+// polls (a poll is a trip to L2, about 0.7 us).
+__device__ __forceinline__ bool group_wait(const unsigned *bar, unsigned target, int polls)
 {
-    for (int i = 0; i < (1 << 22); ++i) {
+    for (int i = 0; i < polls; ++i) {
         unsigned v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         if ((int)(v - target) >= 0)
@@ -376,7 +376,7 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
                 record();  // the step before's
             if (tid == 0) {
                 atomicAdd(&ctl->bar, 1u);
-                if (group_wait(&ctl->bar, (unsigned)(st + 1) * (unsigned)G)) {
+                if (group_wait(&ctl->bar, (unsigned)(st + 1) * (unsigned)G, A.wait_polls)) {
                     sh.step_mseg = __ldcg(&ctl->acc[now].maxseg);
                     sh.step_err = (unsigned)__ldcg(&ctl->acc[now].pad[0]);
                 } else {
@@ -386,7 +386,11 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
         }
         __syncthreads();
         if (sh.gave_up) {
-            // (no copies are in flight: the next step's have not started)
+            // (No copies are in flight: the next step's have not started.)  The
+            // bits stay whatever the recorder does, which may still see the
+            // count complete and record this step: this block's part of the
+            // state is missing, so the simulation is not stepped again, and
+            // the group's buffers, which nobody clears now, are not used again.
             if (tid == 0) {
                 atomicOr(&S.sc->err, SIC_ERR_TIMEOUT);
                 atomicOr(&S.sc->hold, SIC_HOLD_ERROR);
@@ -549,8 +553,10 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
                 sc->step = step0 + st + 1;
                 sc->q_total = qtot;
                 sc->maxseg = mm;
-                sc->err = err;
-                sc->hold = hold;
+                if (err)  // (added: a block that gave up has put its own there)
+                    atomicOr(&sc->err, err);
+                if (hold)
+                    atomicOr(&sc->hold, hold);
                 sc->buf = (unsigned)src;
             }
         }
