@@ -632,6 +632,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsig
     return false;
 }
 
+// A warp that gave up on its copies waits for them once more (as long at most)
+// before it goes on to leave the kernel: they must not land in the shared memory
+// of a block that has exited.
+__device__ __noinline__ void mbar_drain(unsigned long long *bar, unsigned parity)
+{
+    (void)mbar_wait_bounded(bar, parity);
+}
+
 constexpr int kStageBytesU = SIC_STAGE_U_BYTES;
 constexpr int kStageBytesV = SIC_STAGE_V_BYTES;
 constexpr int kStageBytesQ = SIC_STAGE_Q_BYTES;

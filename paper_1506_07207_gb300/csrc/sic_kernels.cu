@@ -429,6 +429,7 @@ __global__ void __launch_bounds__(B, SIC_K1_MIN_BLOCKS) k_step(const LaunchArgs 
                     if (!__all_sync(0xffffffffu, ok)) {
                         // give up (the next item's copies have not started): only count items
                         timed_out = true;
+                        mbar_drain(&sh.mbar[warp][s], ((phase >> s) & 1u) ^ 1u);
                         if (nxt >= 0 && lane == 0)
                             desc_wait();
                         break;

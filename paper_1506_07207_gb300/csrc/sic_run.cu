@@ -166,8 +166,10 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
                     b.nq = Qh[P.next2];
             }
         }
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sh.mbar[warp][0], 0u)))
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sh.mbar[warp][0], 0u))) {
             timed_out = true;
+            mbar_drain(&sh.mbar[warp][0], 0u);
+        }
         __syncwarp();
     }
 
@@ -272,6 +274,7 @@ __device__ __forceinline__ void run_steps(const RunArgs &A, int slot)
             phase ^= 1u << s;
             if (!__all_sync(0xffffffffu, ok)) {  // give up (the next item's copies have not started)
                 timed_out = true;
+                mbar_drain(&sh.mbar[warp][s], ((phase >> s) & 1u) ^ 1u);
                 if (nxt >= 0 && lane == 0)
                     desc_wait();
                 break;
