@@ -272,9 +272,11 @@ int sic_push(sic_sim *sim);
  * by the sheet deposit of Eq. overlap and Eq. rho_sum): gather and push with
  * the current field, deposit every particle of the new positions, solve the
  * field (Sec. 2.1).  Two steps or more are taken many to a kernel launch (a
- * cooperative grid that stays resident); a single step, steps on a stream that
- * is being captured and meshes too large for that take one launch a step, runs
- * of 8 in a replayed graph.
+ * cooperative grid that stays resident); a single step, and simulations too large
+ * for that, take one launch a step, runs of 8 in a replayed graph.  Steps on a
+ * stream that is being captured go into the capture, one launch a step; a step
+ * and a sync come before the first capture, and the captured steps may be
+ * replayed until the simulation is refined or destroyed.
  * n_steps >= 0.  Asynchronous on the simulation's stream: errors found on
  * the device are returned by the next synchronising call (sic_sync,
  * sic_diagnostics, ...).  A held simulation (an error, or a particle past

@@ -759,13 +759,21 @@ void set_schedule(Plan &p, int claim_div, int staging, int claim_min)
 
 constexpr int kStepsALaunch = 256;
 
+// Steps on a stream that is being captured go into the capture one launch each:
+// a graph of one's own can neither be captured nor launched there, and a
+// cooperative grid is not taken into a caller's graph.
+static bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 bool launch_many(Plan &p, int n_steps, cudaStream_t s, cudaError_t &e)
 {
     e = cudaSuccess;
     if (!p.run_grid || n_steps < (p.args.n_slots ? 2 : 1))  // (a single step is as well launched by itself)
         return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    if (capturing(s))
         return false;
     for (int left = n_steps; left > 0 && e == cudaSuccess;) {
         RunArgs a = p.run;
@@ -1297,7 +1305,8 @@ int sic_step(sic_sim *sim, int32_t n_steps)
         if (launch_many(sim->plan, n_steps, sim->stream, e))
             return e == cudaSuccess ? SIC_OK : fail_cuda(sim, e);
     }
-    if (n_steps >= kGraphSteps && !sim->gexec) {
+    const bool graphs = n_steps >= kGraphSteps && !sic_host::capturing(sim->stream);
+    if (graphs && !sim->gexec) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(sim->stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
@@ -1313,7 +1322,7 @@ int sic_step(sic_sim *sim, int32_t n_steps)
         count_launches(-kGraphSteps);  // captured, not run
     }
     int32_t left = n_steps;
-    while (left >= kGraphSteps && sim->gexec) {
+    while (graphs && left >= kGraphSteps) {
         CK(cudaGraphLaunch(sim->gexec, sim->stream));
         count_launches(kGraphSteps);
         left -= kGraphSteps;
@@ -1523,7 +1532,8 @@ int sic_batch_step(sic_batch *b, int32_t n_steps)
             return e == cudaSuccess ? SIC_OK : fail_cuda(sim, e);
     }
     const int launches_per_step = (b->plan[0].mem ? 1 : 0) + (b->plan[1].mem ? 1 : 0);
-    if (n_steps >= kGraphSteps && !b->gexec) {
+    const bool graphs = n_steps >= kGraphSteps && !sic_host::capturing(b->stream);
+    if (graphs && !b->gexec) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
@@ -1539,7 +1549,7 @@ int sic_batch_step(sic_batch *b, int32_t n_steps)
         count_launches(-(int64_t)kGraphSteps * launches_per_step);
     }
     int32_t left = n_steps;
-    while (left >= kGraphSteps && b->gexec) {
+    while (graphs && left >= kGraphSteps) {
         CK(cudaGraphLaunch(b->gexec, b->stream));
         count_launches((int64_t)kGraphSteps * launches_per_step);
         left -= kGraphSteps;
