@@ -548,6 +548,8 @@ void free_plan(Plan &p, cudaStream_t s)
 // a warp on one block, 5.6 on two blocks).
 constexpr int kOneBlockItems = 8;
 
+constexpr int kStepsALaunch = 256;
+
 // The groups of blocks of a launch of many steps (k_run), one per simulation:
 // block_begin[slot], and the grid; 0 when the steps are better launched one
 // by one.  Every group gets a block, and the rest go one by one to the
@@ -566,9 +568,16 @@ constexpr int kOneBlockItems = 8;
 constexpr int kMostRounds = 28;
 constexpr int kMostRoundsBatch = 8;
 
+// Steps that one launch of k_run takes at most.  SIC_STEPS_A_LAUNCH, a test knob
+// read when a plan is built, lowers it: at 1 every step is a launch of k_step (the
+// way of simulations too large for k_run), whatever the sizes.
+static int steps_a_launch() { return std::min(kStepsALaunch, env_int("SIC_STEPS_A_LAUNCH", kStepsALaunch)); }
+
 static int split_blocks(sic_sim *const *sims, int n, int nx_max, int charges, bool gen,
                         std::vector<int32_t> &block_begin)
 {
+    if (steps_a_launch() < 2)
+        return 0;
     const int per_sm = run_blocks_per_sm(nx_max, charges, gen);
     // (SIC_GRID: the test knob of build_plan)
     const int most = std::min(num_sms() * per_sm, std::max(n, env_int("SIC_GRID", num_sms() * per_sm)));
@@ -665,6 +674,7 @@ cudaError_t build_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s)
         gen = gen || sims[slot]->deposit != SIC_DEPOSIT_BOX;
     std::vector<int32_t> block_begin;
     p.run_grid = n == 1 ? split_blocks(sims, n, nx_max, per_q ? 1 : 0, gen, block_begin) : 0;
+    p.run_steps = steps_a_launch();
     p.run_charges = per_q ? 1 : 0;
     p.run_gen = gen;
     Layout lay;
@@ -724,6 +734,7 @@ cudaError_t build_many_plan(Plan &p, sic_sim *const *sims, int n, cudaStream_t s
     p.run_gen = gen;
     std::vector<int32_t> block_begin;
     p.run_grid = split_blocks(sims, n, nx_max, p.run_charges, gen, block_begin);
+    p.run_steps = steps_a_launch();
     if (!p.run_grid)
         return cudaSuccess;
     Layout lay;
@@ -757,8 +768,6 @@ void set_schedule(Plan &p, int claim_div, int staging, int claim_min)
     p.args.claim_min = std::max(1, claim_min);
 }
 
-constexpr int kStepsALaunch = 256;
-
 // Steps on a stream that is being captured go into the capture one launch each:
 // a graph of one's own can neither be captured nor launched there, and a
 // cooperative grid is not taken into a caller's graph.
@@ -777,7 +786,7 @@ bool launch_many(Plan &p, int n_steps, cudaStream_t s, cudaError_t &e)
         return false;
     for (int left = n_steps; left > 0 && e == cudaSuccess;) {
         RunArgs a = p.run;
-        a.n_steps = std::min(left, kStepsALaunch);
+        a.n_steps = std::min(left, p.run_steps);
         e = launch_run_kernel(a, p.run_grid, p.run_charges, p.run_gen, s);
         if (left == n_steps && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
             cudaGetLastError();  // not on this device: one launch a step from now on

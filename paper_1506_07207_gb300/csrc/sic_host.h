@@ -20,6 +20,7 @@ struct Plan {
     bool per_q = false;
     RunArgs run{};       // many steps in one launch (run_grid 0: not for this plan)
     int run_grid = 0;
+    int run_steps = 0;   // steps a launch at most
     int run_charges = 0;
     bool run_gen = false;
 };
