@@ -311,11 +311,15 @@ int sic_batch_step(sic_batch *batch, int32_t n_steps);
  * claim, 1, 2 or 4 items; staging of the items through shared memory
  * automatic, off, or on whenever it fits) is timed with CUDA events on
  * steps_each real steps (after one untimed step), and the fastest is kept
- * for the batch's later steps.  The schedule never changes results (they
- * are bit-identical under every choice), so the timed steps are ordinary
- * steps: the call advances every member by SIC_AUTOTUNE_CANDIDATES
- * (steps_each + 1) steps.  *claim_div, *staging and *claim_min (nullable)
- * get the choice (staging: 0 automatic, 1 off, 2 on).  steps_each >= 1.
+ * for the batch's later steps.  In a batch that takes many steps to a launch
+ * these launches are the last candidate: while they are the fastest they stay,
+ * and the schedule kept is that of steps of one launch each (on a stream that is
+ * being captured); else the batch takes one launch a step from then on.  The
+ * schedule never changes results (they are bit-identical under every choice), so
+ * the timed steps are ordinary steps: the call advances every member by
+ * SIC_AUTOTUNE_CANDIDATES (steps_each + 1) steps.  *claim_div, *staging and
+ * *claim_min (nullable) get the choice of schedule (staging: 0 automatic, 1 off,
+ * 2 on).  steps_each >= 1.
  */
 #define SIC_AUTOTUNE_CANDIDATES 10
 int sic_batch_autotune(sic_batch *batch, int32_t steps_each, int32_t *claim_div, int32_t *staging,

@@ -1589,17 +1589,32 @@ int sic_batch_autotune(sic_batch *b, int32_t steps_each, int32_t *claim_div, int
         return SIC_ECUDA;
     }
     int best = 0;
-    float best_ms = 0.f;
+    float best_ms = 0.f, many_ms = 0.f;
+    bool many = false;
     cudaError_t e = cudaSuccess;
     for (int c = 0; c < n_cand && e == cudaSuccess; ++c) {
         for (auto &p : b->plan)
             if (p.mem)
                 set_schedule(p, cand[c][0], cand[c][1], cand[c][2]);
-        e = batch_launch(b);  // settles caches and the function attributes
+        // a batch that takes launches of many steps: these are timed in the
+        // last schedule's place, as sic_batch_step launches them
+        many = c + 1 == n_cand && b->many.run_grid > 0;
+        auto steps = [&](int n) {
+            cudaError_t r = cudaSuccess;
+            if (many) {
+                many = sic_host::launch_many(b->many, n, b->stream, r);
+                if (many)
+                    return r;  // (else the device does not take them: the schedule after all)
+            }
+            for (int i = 0; i < n && r == cudaSuccess; ++i)
+                r = batch_launch(b);
+            return r;
+        };
+        e = steps(1);  // settles caches and the function attributes
         if (e == cudaSuccess)
             e = cudaEventRecord(ev[0], b->stream);
-        for (int i = 0; i < steps_each && e == cudaSuccess; ++i)
-            e = batch_launch(b);
+        if (e == cudaSuccess)
+            e = steps(steps_each);
         if (e == cudaSuccess)
             e = cudaEventRecord(ev[1], b->stream);
         if (e == cudaSuccess)
@@ -1607,7 +1622,9 @@ int sic_batch_autotune(sic_batch *b, int32_t steps_each, int32_t *claim_div, int
         float ms = 0.f;
         if (e == cudaSuccess)
             e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-        if (e == cudaSuccess && (c == 0 || ms < best_ms)) {
+        if (e == cudaSuccess && many) {
+            many_ms = ms;
+        } else if (e == cudaSuccess && (c == 0 || ms < best_ms)) {
             best = c;
             best_ms = ms;
         }
@@ -1619,6 +1636,10 @@ int sic_batch_autotune(sic_batch *b, int32_t steps_each, int32_t *claim_div, int
     for (auto &p : b->plan)
         if (p.mem)
             set_schedule(p, cand[best][0], cand[best][1], cand[best][2]);
+    if (many && best_ms < many_ms) {  // one launch a step is faster
+        sic_host::free_plan(b->many, b->stream);
+        b->many.run_grid = 0;
+    }
     if (claim_div)
         *claim_div = cand[best][0];
     if (staging)

@@ -211,3 +211,31 @@ def test_large_meshes_take_many_steps(sic, one_step_a_launch, knob, nx):
     finally:
         for s in ones + alls + members:
             s.sic_destroy()
+
+
+def test_autotune_times_launches_of_many_steps_too(sic, one_step_a_launch):
+    """A small batch (its steps are launch latencies, so that many to a launch take half
+    the time): the launches of many steps are one of the candidates, in one launch each for
+    the untimed and the timed steps, and stay.  A batch that does not take them times
+    schedules only.  Both advance by the same steps, to the same bits."""
+    probs = [inputs.landau(0.1, 0.4, 64, 16, 300, t_end=20.0), inputs.landau(0.1, 0.5, 128, 8, 600, t_end=20.0)]
+    n, each = sic.SIC_AUTOTUNE_CANDIDATES, 16
+    got = []
+    for knob in ("256", "1"):
+        one_step_a_launch.setenv("SIC_STEPS_A_LAUNCH", knob)
+        sims = [sic.Sim.from_problem(p, history_len=300) for p in probs]
+        b = sic.Batch(sims)
+        try:
+            tuned = _launches(sic, lambda: b.sic_batch_autotune(each))
+            assert tuned == ((n - 1) * (each + 1) + 2 if knob == "256" else n * (each + 1))
+            assert _launches(sic, lambda: b.sic_batch_step(12)) == (1 if knob == "256" else 12)
+            b.sic_batch_destroy()
+            assert all(s.sic_diagnostics()["step"] == n * (each + 1) + 12 for s in sims)
+            got.append([(*s.sic_get_state(), s.sic_history(300)) for s in sims])
+        finally:
+            b.sic_batch_destroy()
+            for s in sims:
+                s.sic_destroy()
+    for a, b in zip(*got):
+        for x, y in zip(a, b):
+            np.testing.assert_array_equal(x, y)
