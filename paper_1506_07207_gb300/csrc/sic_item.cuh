@@ -933,6 +933,7 @@ __device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int 
     unsigned pend = 0;  // charge waiting for cell c (below 2^32: at most 9 shares of 2^28)
     int c = jn[0];
     int done = 0;       // segments of the lane dealt with
+    bool spread = false;  // the item's particles are dealt over the lanes
     if (who) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -947,13 +948,35 @@ __device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int 
         }
         if (PER_Q)
             tab[kTabWords + 32 * R + lane] = qsum;
+        // A short item (a short sheet, or what is left of one) leaves most lanes
+        // without a tracer and the others a long loop each: where half of its
+        // particles or more cross, they are dealt over all lanes instead, those
+        // inside a cell too, each adding its own shares.  Single steps of one
+        // launch, us with the loops and this: 172 sheets of up to 60 tracers on
+        // 114 cells 20.7 and 15.1, 2000 of up to 100 on 500 28.3 and 20.8 (one
+        // launch for many 14.2 and 11.5), 2048 of 64 on 1024 25.5 and 19.8.  At 120
+        // tracers on 64 cells, 40 % of them crossing, 15.8 with the loops: the
+        // lanes inside a cell would all add into the same few words.  Up to 128
+        // particles, four a lane: up to 64 only, 500 sheets of up to 100 on 2048
+        // cells took 31.6 and not 25.5.
+        if (!FULL) {
+            spread = nseg_item <= 4 * 32 && 2 * (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(cross)) >= nseg_item;
+            if (spread) {
+                const int left = nseg_item - lane;
+                cross = left > 0 ? (2u << ((left - 1) >> 5)) - 1u : 0u;
+                __syncwarp();
+            }
+        }
         while (cross) {
             const int k = __ffs(cross) - 1;
             cross &= cross - 1u;
-            const unsigned pa = tab[32 * k + lane], pb = tab[32 * k + 32 + lane];
+            int at = 32 * k + lane;
+            if (!FULL && spread)
+                at = 32 * (lane & (R - 1)) + (at >> 3);
+            const unsigned pa = tab[at], pb = tab[at + 32];
             unsigned qs, before;
             if (PER_Q) {
-                const unsigned q0 = tab[kTabWords + 32 * k + lane], q1 = tab[kTabWords + 32 * k + 32 + lane];
+                const unsigned q0 = tab[kTabWords + at], q1 = tab[kTabWords + at + 32];
                 qs = q1 - q0;
                 before = q0 - tab[kTabWords + 32 * done + lane];
             } else {
@@ -965,6 +988,14 @@ __device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int 
             const int d = (int)(pb - pa);
             const bool back = d < 0;
             const unsigned len = (unsigned)abs(d);
+            if (!FULL && spread) {
+                before = 0u;
+                c = cell_of(cell_coord(pa, nx));
+                if (c == cb && (pb - pa + (1u << 29)) < (1u << 30)) {  // inside its cell
+                    hist.add32(c, qs);
+                    continue;
+                }
+            }
             mlen = max(mlen, len);
             const unsigned la = (back ? pb : pa) * nx4;  // the lower end's fraction of its cell
             const unsigned long long span = (unsigned long long)len * nx4;
@@ -1019,8 +1050,14 @@ __device__ __forceinline__ void deposit_boxes(const unsigned (&u)[R], const int 
             hist.add32(c, pend + before + (back ? rest : F));
             pend = back ? F : rest;
             c = cb;
+            if (!FULL && spread) {
+                hist.add32(c, pend);
+                pend = 0u;
+            }
         }
     }
+    if (!FULL && spread)
+        return;
     // what is left of the lane, in the cell its sheet is in now
     if (PER_Q) {
         const unsigned left = pend + (qsum - (done ? tab[kTabWords + 32 * done + lane] : 0u));
