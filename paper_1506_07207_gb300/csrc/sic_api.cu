@@ -564,9 +564,18 @@ constexpr int kStepsALaunch = 256;
 // 42 and 37, 27 rounds 69 and 69, 55 rounds 112 and 116.  In a batch, blocks
 // do not help another simulation's, so the launch is as slow as the group whose
 // items cost most: 3.4 rounds 24 and 18, 6.7 rounds of 16 simulations 27 and
-// 20, the same half folded 71 and 46, 17 rounds half folded 103 and 115.
+// 20, the same half folded 71 and 46, 17 rounds half folded 103 and 115.  Larger
+// meshes, whose field every block solves, move the lines little: alone 27 rounds
+// on 2048 cells 73.6 and 73.1, on 3000 81.9 and 82.4, on 6000 95 and 92; in a batch
+// 8 rounds on 3000 58 and 52, on 6000 66 and 59.  What moves them is an SM that
+// holds two blocks of k_step and one of k_run, which stages its items (between
+// about 3100 and 4100 cells): on 4096 cells alone 7 rounds 35 and 34, 13 rounds
+// 44 and 47, 27 rounds 66 and 77, in a batch 3 rounds 43 and 32, 6 rounds 46 and
+// 45, 8 rounds 52 and 54.
 constexpr int kMostRounds = 28;
 constexpr int kMostRoundsBatch = 8;
+constexpr int kMostRoundsFewer = 10;  // where the SM holds fewer blocks than of k_step
+constexpr int kMostRoundsBatchFewer = 6;
 
 // Steps that one launch of k_run takes at most.  SIC_STEPS_A_LAUNCH, a test knob
 // read when a plan is built, lowers it: at 1 every step is a launch of k_step (the
@@ -608,7 +617,8 @@ static int split_blocks(sic_sim *const *sims, int n, int nx_max, int charges, bo
     int rounds = 0;
     for (int i = 0; i < n; ++i)
         rounds = std::max(rounds, ((int)sims[i]->items.size() + SIC_K1_WARPS * blocks[i] - 1) / (SIC_K1_WARPS * blocks[i]));
-    if (rounds > (n == 1 ? kMostRounds : kMostRoundsBatch))
+    const bool fewer = per_sm < step_blocks_per_sm(nx_max, MODE_STEP, charges != 0);
+    if (rounds > (n == 1 ? (fewer ? kMostRoundsFewer : kMostRounds) : (fewer ? kMostRoundsBatchFewer : kMostRoundsBatch)))
         return 0;
     block_begin.assign(n + 1, 0);
     for (int i = 0; i < n; ++i)

@@ -239,3 +239,34 @@ def test_autotune_times_launches_of_many_steps_too(sic, one_step_a_launch):
     for a, b in zip(*got):
         for x, y in zip(a, b):
             np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("members,rounds", [(1, 9), (1, 12), (4, 5), (4, 7)])
+@pytest.mark.parametrize("nx", [3000, 4096])
+def test_the_rule_on_rounds_of_items(sic, nx, members, rounds):
+    """Where an SM holds one block of a launch of many steps and two of single steps (4096
+    cells), fewer rounds of items (one per warp) go to launches of many steps; on 3000
+    cells it holds two of each.  Either way: the steps of single launches."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    warps = 8 * sms * (2 if nx == 3000 else 1)
+    sheets = int((rounds - 0.4) * warps / members) // 8        # of 8 items each
+    p = inputs.landau(0.01, 0.5, nx, sheets, 2048, t_end=1.0)
+    ones, many = ([sic.Sim.from_problem(p, history_len=16) for _ in range(members)] for _ in range(2))
+    b = sic.Batch(many) if members > 1 else None
+    try:
+        step = b.sic_batch_step if b else many[0].sic_step
+        takes_many = nx == 3000 or rounds <= (10 if members == 1 else 6)
+        assert _launches(sic, lambda: step(9)) == (1 if takes_many else 9)
+        if b:
+            b.sic_batch_destroy()
+        for s, t in zip(many, ones):
+            for _ in range(9):
+                t.sic_step(1)
+            np.testing.assert_array_equal(s.sic_history(16), t.sic_history(16))
+            np.testing.assert_array_equal(s.sic_deposit()[0], t.sic_deposit()[0])
+    finally:
+        if b:
+            b.sic_batch_destroy()
+        for s in ones + many:
+            s.sic_destroy()
