@@ -27,7 +27,7 @@ in log2 (``inputs.serving_mix``, seed 0x5EC5).
 * ``single_sim``: the two-stream (512 x 16384 = 8,388,608 segments, Nx
   1024), nonlinear Landau (1024 x 4096, Nx 512), linear Landau (256 x 1024,
   Nx 128) and Langmuir (1 x 4096, Nx 64) configurations stepped alone:
-  graphs of 8 steps with a 256 MB L2 flush before each, and single steps
+  8 steps a launch with a 256 MB L2 flush before each, and single steps
   with a flush before each.
 
     python bench.py [--gpus N --steps K --warmup W] [--impl reference]
@@ -130,17 +130,24 @@ class Clocks:
                 "sm_max_mhz": max(mx) if mx else None, "reasons": reasons, "samples": len(rows)}
 
 
+def step_kernel_sha256():
+    """Hash of the sources that the step kernels are compiled from."""
+    import hashlib
+    h = hashlib.sha256()
+    for name in ("sic_kernels.cu", "sic_run.cu", "sic_item.cuh", "sic_internal.h"):
+        with open(os.path.join(ROOT, "paper_1506_07207_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
+
+
 def kernel_traffic(segments):
     """DRAM bytes of one step-kernel launch over `segments` segments, scaled
     from an ncu capture of a smaller case (profiles/k_step_traffic.json), or
-    None when the kernel source changed since that capture."""
-    import hashlib
+    None when a source of the step kernels changed since that capture."""
     path = os.path.join(ROOT, "profiles", "k_step_traffic.json")
-    src = os.path.join(ROOT, "paper_1506_07207_gb300", "csrc", "sic_kernels.cu")
     try:
         d = json.load(open(path))
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()
-        if d.get("kernel_sha256") != sha:
+        if d.get("kernel_sha256") != step_kernel_sha256():
             return None
         return float(d["dram_bytes_per_segment"]) * segments
     except Exception:
@@ -278,8 +285,8 @@ def single_sim(torch, Sim, steps, warmup):
     """One simulation alone: the two-stream and nonlinear Landau
     configurations (the roofline applies), and the linear Landau and Langmuir
     ones (small: bound by launch and latency, absolute times only).  Two
-    timings each: steps as a user runs them (sic_step of 8 steps, one CUDA
-    graph, the L2 flushed before every group of 8), and one step per call with
+    timings each: steps as a user runs them (sic_step of 8 steps, one
+    launch, the L2 flushed before every group of 8), and one step per call with
     the L2 flushed before every step."""
     from paper_1506_07207_gb300 import inputs
     peak, _ = peaks()
@@ -316,7 +323,7 @@ def single_sim(torch, Sim, steps, warmup):
                      "achieved_gbs": gbs,
                      "roofline_frac": gbs / peak if name in ("two_stream", "landau_nonlinear") else None,
                      "ms_per_step_single_launch": one * 1e3,
-                     "timing": "sic_step(8) (one graph of 8 steps) after a 256 MB L2 flush, per step; "
+                     "timing": "sic_step(8) (8 steps in one launch) after a 256 MB L2 flush, per step; "
                                "single launch: sic_step(1) after a flush"}
     return out
 
@@ -404,7 +411,7 @@ def late_states(torch, Sim, groups=4):
 
 def profile_case(torch, Sim, name):
     """The case of the late-state ncu capture: the state of late_states, then
-    two steps inside an NVTX range named "late"."""
+    two steps (one launch of k_run) inside an NVTX range named "late"."""
     p, pre = late_problem(name)
     sim = Sim.from_problem(p, history_len=8)
     sim.sic_run(pre)

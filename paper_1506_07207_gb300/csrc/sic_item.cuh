@@ -397,8 +397,8 @@ __device__ __forceinline__ float pl_kappa(long long up, long long ua, long long 
 // and taking its parameters from the owner: on folded sheets particles range
 // from two cells to half the box, and a loop per lane (or a warp per long
 // particle) left most lanes idle for a chain of divisions and conversions.
-// A step of 256 x 2048 folded tracers
-// on 256 cells takes 72 us, 120 us with those loops.
+// A step of 256 x 2048 folded tracers on 256 cells takes 71 us, 122 us with those
+// loops (42 us of many steps a launch).
 __device__ __forceinline__ void emit_linear(int jl, unsigned la, float inv, int q, float kappa, int n, int nx,
                                             const Hist &hist)
 {
@@ -907,8 +907,9 @@ __device__ void add_diff_prefix(const Hist &hist, const Hist &diff, int nx, Shar
 // crossing make no commit: the lane with a crossing before them takes their
 // segments into its last one (they lie in one cell), which also spares
 // the adds of many lanes into one word.  No list of the crossing ones is made
-// and no lane works for another.  Against per-cell counts and a warp-wide task
-// list for the crossing ones (us per step, before and after): 4.2 M folded
+// and no lane works for another, but in short items (below).  Against per-cell
+// counts and a warp-wide task list for the crossing ones (us per step, before and
+// after): 4.2 M folded
 // tracers 72 and 51, 2.3 M folded 50 and 34, 8.4 M quiet 43 and 41; a batch of
 // 66 M quiet 278 and 246.  (With the whole cells through the general
 // range_add, a call of 64-bit adds: 60, 42.)

@@ -942,7 +942,7 @@ namespace {
 // into FP64 by their bits, and the reciprocal of the length is one
 // third-order step from the FP32 one.  The diagnostics of 512 x 2048 folded
 // tracers on 512 cells (both orders, a deposit, the field and two spectra) take
-// 0.47 ms, of which the moments 98 and 199 us as calls; 0.72 ms with one mesh
+// 0.46 ms, of which the moments 88 and 186 us as calls; 0.72 ms with one mesh
 // for all blocks, 1.59 ms with every cell's share worked out as well, 49.5 ms
 // with one thread per work item.
 constexpr int kMomentCells = 8;
