@@ -218,8 +218,8 @@ def test_autotune_times_launches_of_many_steps_too(sic, one_step_a_launch):
     the time): the launches of many steps are one of the candidates, in one launch each for
     the untimed and the timed steps, and stay.  A batch that does not take them times
     schedules only.  Both advance by the same steps, to the same bits."""
-    probs = [inputs.landau(0.1, 0.4, 64, 16, 300, t_end=20.0), inputs.landau(0.1, 0.5, 128, 8, 600, t_end=20.0)]
-    n, each = sic.SIC_AUTOTUNE_CANDIDATES, 16
+    probs = [inputs.landau(0.1, 0.4, 64, 16, 300, dt=1e-3), inputs.landau(0.1, 0.5, 128, 8, 600, dt=1e-3)]
+    n, each = sic.SIC_AUTOTUNE_CANDIDATES, 100  # (0.6 and 1.2 ms: far more than a hiccup of the host)
     got = []
     for knob in ("256", "1"):
         one_step_a_launch.setenv("SIC_STEPS_A_LAUNCH", knob)
